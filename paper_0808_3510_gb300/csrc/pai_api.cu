@@ -353,7 +353,6 @@ pai_status enqueue_row(pai_plan_s* P, bool adjoint, cudaStream_t s, int threads,
     smem = P->smem_adj3;
     ctas = P->spread_mode == 3 ? P->ctas_adj3 : P->ctas_adj4;
   }
-  PAI_CUDA(cudaMemsetAsync(L.counter, 0, sizeof(int), s));
   cudaError_t e = adjoint ? launch_row_adjoint(L, P->poly, threads, ctas, smem, s, zf)
                           : launch_row_forward(L, P->poly, threads, ctas, smem, s, zf);
   return cuda_status(e);
@@ -808,6 +807,7 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
   PAI_TRY(plan_malloc(P, (void**)&P->d_tw, tw.size() * sizeof(float2)));
   PAI_TRY(plan_malloc(P, (void**)&P->d_problems, count * sizeof(RowProblem)));
   PAI_TRY(plan_malloc(P, (void**)&P->d_counter, 4 * sizeof(int)));
+  PAI_CUDA(cudaMemset(P->d_counter, 0, 4 * sizeof(int)));
   PAI_CUDA(cudaMemcpy(P->d_tables, tables.data(), tab_off * sizeof(float), cudaMemcpyHostToDevice));
   PAI_CUDA(cudaMemcpy(P->d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice));
 
