@@ -303,11 +303,13 @@ pai_status pai_window_probe(int H, double beta, double c, int n, const double* y
  * box.
  *
  * pai_forward_plan: g as for pai_plan (method KB or TSINC); box extents up to
- * 16384 laterally and 8192 in depth (PAI_ERR_UNSUPPORTED beyond); allocates
- * the box buffers (4 (bx by bz + bx by nt) bytes) besides the plan's own.
+ * 16384 laterally and 8192 in depth (PAI_ERR_UNSUPPORTED beyond); the
+ * box itself is never stored (the plan's spectra are 8 bytes x the box's lateral
+ * rows x about (max(nt, nz) + bz/2)).
  * The returned plan accepts pai_forward_model, pai_forward_box, pai_get_info
  * (describing the box geometry), pai_set_stream, pai_launch_count,
- * pai_profile_stages with adjoint = 1 (box-sized buffers) and pai_destroy;
+ * pai_profile_stages with adjoint = 1 (d_in image-shaped, d_out data-shaped)
+ * and pai_destroy;
  * the other calls return PAI_ERR_INVALID_ARG.
  * pai_forward_model: d_f device FP32 image [nx][ny][nz], read only; d_p
  * device FP32 data [nx][ny][nt], overwritten.  Asynchronous on the plan's
@@ -348,8 +350,7 @@ pai_status pai_forward_box(pai_plan_t plan, int* bx, int* by, int* bz);
  * PAI_ERR_INVALID_ARG; batched plans return PAI_ERR_UNSUPPORTED.  Computes
  * the table, uploads it into plan-owned device memory and waits for the
  * upload.  A forward-model plan with a cutoff returns w_cut * (Q f) from
- * pai_forward_model: the weight is applied by the kernel that copies the
- * detector rows out of the box, at no extra memory traffic.
+ * pai_forward_model: the weight is applied in place to the samples it changes.
  *
  * pai_cutoff: d_out = w_cut * d_in over the plan's data grid [nx][ny][nt]
  * (device FP32, contiguous).  d_in == d_out (in place) touches only the

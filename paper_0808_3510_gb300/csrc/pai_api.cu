@@ -122,8 +122,6 @@ struct pai_plan_s {
   // the padded box; the image / detector geometry and the box buffers
   bool qmode = false;
   pai_geometry qimg{};
-  float* d_qin = nullptr;   // box image
-  float* d_qout = nullptr;  // box data
   // data cutoff w_cut (pai_set_cutoff): weight table on the device
   float* d_cut = nullptr;
   int cut_R = 0;
@@ -280,8 +278,6 @@ void release(pai_plan_s* P) {
   if (P->stream) cudaStreamSynchronize(P->stream);
   if (P->s_up) cudaStreamSynchronize(P->s_up);
   if (P->s_down) cudaStreamSynchronize(P->s_down);
-  cudaFree(P->d_qin);
-  cudaFree(P->d_qout);
   cudaFree(P->d_cut);
   for (int k = 0; k < 2; ++k) {
     cudaFree(P->d_pipe_in[k]);
@@ -397,8 +393,35 @@ pai_status enqueue_inverse(pai_plan_s* P, const ProblemHost& p, float* d_f, cuda
   return fft_status(cufftExecC2R(p.img_c2r, (cufftComplex*)(P->d_fh + p.fh_off), d_f + p.img_off));
 }
 
+// First and last stages of the forward model: the box is never in memory.  The
+// image's own layers are transformed laterally with zeros read for the rest of
+// the box, then each lateral row along depth, folded to the sums the node pairs
+// carry (launch_rows_fold); behind the row kernel only the detectors' rows are
+// transformed back.  (Padding, transforming and cropping the whole box took
+// 1.39 of 2.67 ms for a 128^3 volume in its 512^3 box.)
+pai_status enqueue_model_first(pai_plan_s* P, const ProblemHost& p, const float* d_f, cudaStream_t s) {
+  const pai_geometry &b = p.g, &gi = P->qimg;
+  const float2* tw = P->d_tw;
+  if (b.dim == 2) {
+    PAI_CUDA(launch_lateral_r2c(d_f, P->d_pt, b.nx, gi.nz, 1, tw, P->TW / b.nx, s, gi.nx));
+  } else {
+    PAI_CUDA(launch_lateral_r2c(d_f, P->d_fh, b.ny, gi.nz, gi.nx, tw, P->TW / b.ny, s, gi.ny));
+    PAI_CUDA(launch_lateral_c2c(P->d_fh, P->d_pt, b.nx, (b.ny / 2 + 1) * gi.nz, 1, false, tw, P->TW / b.nx, s, gi.nx));
+  }
+  return cuda_status(launch_rows_fold(P->d_pt, gi.nz, P->d_fh, b.nz, p.rows, tw, P->TW / b.nz, s));
+}
+
+pai_status enqueue_model_last(pai_plan_s* P, const ProblemHost& p, float* d_p, cudaStream_t s) {
+  const pai_geometry &b = p.g, &gi = P->qimg;
+  const float2* tw = P->d_tw;
+  if (b.dim == 2) return cuda_status(launch_lateral_c2r(P->d_pt, d_p, b.nx, b.nt, 1, tw, P->TW / b.nx, s, gi.nx));
+  PAI_CUDA(launch_lateral_c2c(P->d_pt, P->d_pt, b.nx, (b.ny / 2 + 1) * b.nt, 1, true, tw, P->TW / b.nx, s, gi.nx));
+  return cuda_status(launch_lateral_c2r(P->d_pt, d_p, b.ny, b.nt, gi.nx, tw, P->TW / b.ny, s, gi.ny));
+}
+
 // First and last stages of the adjoint for problem p.
 pai_status enqueue_adj_first(pai_plan_s* P, const ProblemHost& p, const float* d_h, cudaStream_t s) {
+  if (P->qmode) return enqueue_model_first(P, p, d_h, s);
   if (P->zf_adj) {
     PAI_TRY(own_lateral_fwd(P, p, d_h + p.img_off, P->d_fh + p.fh_off, p.g.nz, s));
     return cuda_status(launch_rows_c2c(P->d_fh + p.fh_off, p.g.nz, p.rows, false, P->d_tw, P->TW / p.g.nz, s));
@@ -407,6 +430,7 @@ pai_status enqueue_adj_first(pai_plan_s* P, const ProblemHost& p, const float* d
 }
 
 pai_status enqueue_adj_last(pai_plan_s* P, const ProblemHost& p, float* d_pbar, cudaStream_t s) {
+  if (P->qmode) return enqueue_model_last(P, p, d_pbar, s);
   if (P->zf_adj) return own_lateral_inv(P, p, P->d_pt + p.pt_off, d_pbar + p.data_off, p.g.nt, s);
   return fft_status(cufftExecC2R(p.lat_c2r, (cufftComplex*)(P->d_pt + p.pt_off), d_pbar + p.data_off));
 }
@@ -548,8 +572,11 @@ std::string wisdom_key(int device, const pai_geometry* gs, int count) {
   return k;
 }
 
-// Plan construction shared by pai_plan and pai_plan_batched.
-pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_s** out, bool qmode = false) {
+// Plan construction shared by pai_plan and pai_plan_batched, and by
+// pai_forward_plan (qimg: the image's geometry, gs its padded box).
+pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_s** out,
+                      const pai_geometry* qimg = nullptr) {
+  const bool qmode = qimg != nullptr;
   if (!gs || !out || count < 1) return PAI_ERR_INVALID_ARG;
   for (int i = 0; i < count; ++i) PAI_TRY(validate(gs[i]));
   for (int i = 1; i < count; ++i)
@@ -744,6 +771,7 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     P->zf = zf;
     P->zf_adj = zf;
     P->qmode = qmode;
+    if (qmode) P->qimg = *qimg;
   }
 
   // ---- layout -------------------------------------------------------------
@@ -761,9 +789,17 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     p.fh_off = fh_off;
     data_off += p.data_len();
     img_off += p.img_len();
-    pt_off += (size_t)p.rows * p.g.nt;
-    // half image spectrum [n1 n2][lz] (non-fused row kernel) or depth rows [rows][nz] (fused)
-    fh_off += std::max((size_t)p.n1 * p.n2 * p.lz, (size_t)p.rows * p.g.nz);
+    if (qmode) {
+      // forward model: pt holds the lateral spectra of the image's layers, then the row kernel's output; fh the
+      // y-transformed layers (3-D), then the folded depth spectra [rows][nz/2 + 2]
+      pt_off += (size_t)p.rows * std::max(p.g.nt, qimg->nz);
+      fh_off += std::max((size_t)p.rows * (p.g.nz / 2 + 2),
+                         p.g.dim == 3 ? (size_t)qimg->nx * (p.g.ny / 2 + 1) * qimg->nz : 0);
+    } else {
+      pt_off += (size_t)p.rows * p.g.nt;
+      // half image spectrum [n1 n2][lz] (non-fused row kernel) or depth rows [rows][nz] (fused)
+      fh_off += std::max((size_t)p.n1 * p.n2 * p.lz, (size_t)p.rows * p.g.nz);
+    }
     p.pre_off = tab_off;
     tab_off = align4(tab_off + p.g.nt);
     p.rowS_off = tab_off;
@@ -824,6 +860,7 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     r.paired = p.paired ? 1 : 0;
     if (qmode) {
       r.qmode = 1;
+      r.zstride = p.g.nz / 2 + 2;
       r.wscale = (float)(0.5 / ((double)r.n1 * r.n2 * p.g.nz));
     }
   }
@@ -1303,20 +1340,6 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
   return PAI_OK;
 }
 
-// Zero-padded copy of an image [nx][ny][nz] into the box [bx][by][bz]
-// (the image at the box origin, zeros elsewhere); z fastest, coalesced.
-__global__ void pad_box_kernel(const float* __restrict__ in, float* __restrict__ out, int nx, int ny, int nz,
-                               int by, int bz, long long total) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int z = (int)(i % bz);
-    const long long xy = i / bz;
-    const int y = (int)(xy % by);
-    const int x = (int)(xy / by);
-    out[i] = (x < nx && y < ny && z < nz) ? in[((size_t)x * ny + y) * nz + z] : 0.0f;
-  }
-}
-
 // Box of the discrete forward model along one axis: room for the image and for
 // the distance sound travels in the recorded time, so that no periodic image of
 // the object reaches the detectors within it (next power of two).
@@ -1634,16 +1657,7 @@ pai_status pai_forward_plan(const pai_geometry* g, void* cuda_stream, pai_plan_t
   gb.nz = forward_box_extent(gi.nz, gi.dz, gi);
   if (gb.nx > 16384 || gb.ny > 16384 || gb.nz > 8192) return PAI_ERR_UNSUPPORTED;
   pai_plan_s* P = nullptr;
-  PAI_TRY(build_plan(&gb, 1, cuda_stream, &P, true));
-  P->qimg = gi;
-  const size_t box_img = (size_t)gb.nx * gb.ny * gb.nz, box_dat = (size_t)gb.nx * gb.ny * gb.nt;
-  pai_status st = plan_malloc(P, (void**)&P->d_qin, box_img * sizeof(float));
-  if (st == PAI_OK) st = plan_malloc(P, (void**)&P->d_qout, box_dat * sizeof(float));
-  if (st != PAI_OK) {
-    release(P);
-    return st == PAI_ERR_CUDA ? PAI_ERR_OOM : st;
-  }
-  P->ws_bytes = (size_t)P->alloc_used;
+  PAI_TRY(build_plan(&gb, 1, cuda_stream, &P, &gi));
   *out = P;
   return PAI_OK;
 }
@@ -1664,28 +1678,19 @@ pai_status pai_forward_model(pai_plan_t plan, const float* d_f, float* d_p) {
   cudaGetDevice(&prev);
   if (prev != plan->device) cudaSetDevice(plan->device);
   const pai_geometry& gi = plan->qimg;
-  const pai_geometry& gb = plan->probs[0].g;
-  const int by = gb.dim == 3 ? gb.ny : 1, ny = gi.dim == 3 ? gi.ny : 1;
-  const long long total = (long long)gb.nx * by * gb.nz;
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, plan->device);
-  const long long want = (total + 255) / 256;
-  const int blocks = (int)std::min<long long>(want, (long long)std::max(sms, 1) * 16);
-  pad_box_kernel<<<blocks, 256, 0, plan->stream>>>(d_f, plan->d_qin, gi.nx, ny, gi.nz, by, gb.nz, total);
-  pai_status st = cuda_status(cudaGetLastError());
-  if (st == PAI_OK) st = run(plan, plan->d_qin, plan->d_qout, true);
+  const int ny = gi.dim == 3 ? gi.ny : 1;
+  // plain launches, not a graph kept per pointer pair: four to six kernels of a
+  // call that takes longer than their launches, and no capture on new buffers
+  pai_status st = enqueue_adjoint(plan, d_f, d_p, plan->stream);
+  if (st == PAI_OK) plan->own_kernels += plan->own_kernels_per_adj;
   if (st == PAI_OK && plan->d_cut) {
-    // the data model g = w_cut * (Q f): the weight applied while the detector rows leave the box
-    CutoffLaunch a{plan->d_qout, d_p, plan->d_cut, gi.nx, ny, gi.nt, by, plan->cut_R, gi.dim};
+    // the data model g = w_cut * (Q f): only the samples near the faces are touched
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, plan->device);
+    CutoffLaunch a{d_p, d_p, plan->d_cut, gi.nx, ny, gi.nt, ny, plan->cut_R, gi.dim};
     st = cuda_status(launch_cutoff(a, plan->stream, sms));
     if (st == PAI_OK) plan->own_kernels += 1;
-  } else if (st == PAI_OK) {
-    // detectors x < nx (and y < ny) of the box data [bx][by][nt]
-    const size_t row = (size_t)ny * gi.nt * sizeof(float), pitch = (size_t)by * gi.nt * sizeof(float);
-    st = cuda_status(cudaMemcpy2DAsync(d_p, row, plan->d_qout, pitch, row, gi.nx, cudaMemcpyDeviceToDevice,
-                                       plan->stream));
   }
-  if (st == PAI_OK) plan->own_kernels += 1;  // the pad kernel (the rest is counted by run)
   if (prev != plan->device) cudaSetDevice(prev);
   return st;
 }

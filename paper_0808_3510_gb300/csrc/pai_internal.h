@@ -69,6 +69,8 @@ struct RowProblem {
   int nzshift;             // log2(nz) when nz is a power of two, else 0
   int method;              // PAI_METHOD_*
   int qmode;               // adjoint kernel evaluates the discrete forward model (depth-row layout only)
+  int zstride;             // depth-row layout: complex values from one row to the next (nz; in qmode
+                           // the rows hold c_j, j = 0..nz/2, nz/2 + 2 values apart)
   int paired;              // 2-D, forward: pt holds Z[k][m] (k < nx = n2, m < nt/2, row stride nt/2), the
                            // lateral DFT of the sample pairs p[x][2m] + i p[x][2m+1]; the forward row kernel
                            // separates row k's samples from Z[k] and Z[nx - k]
@@ -170,15 +172,21 @@ size_t row_fft_region_bytes(int threads, int M);
 
 // FFTs along a strided axis of A[outer][L][C] for power-of-two L, pai_lateral.cu.
 bool lateral_supported(int L, int C);
+// n (0: L): only the first n of the L points of the axis exist on the side named real (c2c: on the input of the
+// forward, the output of the inverse transform): A[outer][n][C]; the others are zeros (input) or not wanted (output).
 cudaError_t launch_lateral_r2c(const float* in, float2* out, int L, int C, int outer, const float2* tw, int twstride,
-                               cudaStream_t s);
+                               cudaStream_t s, int n = 0);
 cudaError_t launch_lateral_c2r(const float2* in, float* out, int L, int C, int outer, const float2* tw, int twstride,
-                               cudaStream_t s);
+                               cudaStream_t s, int n = 0);
 cudaError_t launch_lateral_c2c(const float2* in, float2* out, int L, int C, int outer, bool inverse, const float2* tw,
-                               int twstride, cudaStream_t s);
+                               int twstride, cudaStream_t s, int n = 0);
 // In-place FFT of `rows` contiguous complex lines of power-of-two length L (32 <= L <= 16384).
 cudaError_t launch_rows_c2c(float2* data, int L, int rows, bool inverse, const float2* tw, int twstride,
                             cudaStream_t s);
+// Forward FFT of `rows` lines in[row][n] zero-padded to length L, folded: out[row][j] = F[j] + F[L - j] for
+// 0 < j < L/2, F[0] and F[L/2] alone (j = 0..L/2; out lines are L/2 + 2 values apart).
+cudaError_t launch_rows_fold(const float2* in, int n, float2* out, int L, int rows, const float2* tw, int twstride,
+                             cudaStream_t s);
 // kind: 0 forward row kernel, 1 adjoint row kernel, 2 adjoint row kernel with the pair spread, 3 forward row
 // kernel for launches with problems in the paired layout, 4 adjoint with the atomic pair spread
 int row_kernel_max_ctas_per_sm(int kind, int threads, size_t smem, int H, bool zf = false);

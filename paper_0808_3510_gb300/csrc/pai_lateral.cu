@@ -37,10 +37,26 @@ __device__ __forceinline__ void first_pass_regs(float2* Z, float2 (&z)[kElemsPer
   for (int r = 0; r < kElemsPerThread; ++r) Z[PADI(x0 * kElemsPerThread + r)] = z[r];
 }
 
-template <int KIND, int FP>
+// Two adjacent floats, one load when they start on an 8-byte boundary (pairs).
+template <bool CHECK>
+__device__ __forceinline__ float2 ldg_pair(const float2* p, int pairs) {
+  if (!CHECK || pairs) return __ldg(p);
+  const float* q = reinterpret_cast<const float*>(p);
+  return make_float2(__ldg(q), __ldg(q + 1));
+}
+
+// PRUNED: only the first n of the L points exist on the real side (R2C, C2R)
+// or on the input of the C2C / the output of the inverse C2C; the others are
+// zeros, or are not stored.  The forward model's box is two to four times the
+// image per axis, so most of its traffic is such points.  (Compiled apart: the
+// full kernel keeps its loads without the extra predicate.)  pairs = 0: the
+// real buffer is only 4-byte aligned (the forward model takes such buffers;
+// the plans' other calls ask for 8 bytes), its floats move one at a time.
+template <int KIND, int FP, bool PRUNED>
 __global__ void __launch_bounds__(1024) lateral_kernel(const void* vin, void* vout, int L,
                                                        int mshift, int C, long long in_outer, long long out_outer,
-                                                       const float2* __restrict__ tw, int twstride) {
+                                                       const float2* __restrict__ tw, int twstride, int n,
+                                                       int pairs) {
   extern __shared__ float2 smem[];
   constexpr bool kInv = (KIND == kLatC2R || KIND == kLatC2CInv);
   const int tpr = L / kElemsPerThread;
@@ -64,7 +80,8 @@ __global__ void __launch_bounds__(1024) lateral_kernel(const void* vin, void* vo
     float2 z[kElemsPerThread];
 #pragma unroll
     for (int i = 0; i < kElemsPerThread; ++i)
-      z[i] = live ? __ldg(src + (size_t)i * xs * (C / 2)) : make_float2(0.f, 0.f);
+      z[i] = live && (!PRUNED || x0 + i * xs < n) ? ldg_pair<PRUNED>(src + (size_t)i * xs * (C / 2), pairs)
+                                                  : make_float2(0.f, 0.f);
     first_pass_regs<false>(Z, z, x0);
   } else if (KIND == kLatC2C || KIND == kLatC2CInv) {
     const float2* in = static_cast<const float2*>(vin) + ob * in_outer;
@@ -73,7 +90,7 @@ __global__ void __launch_bounds__(1024) lateral_kernel(const void* vin, void* vo
     float2 z[kElemsPerThread];
 #pragma unroll
     for (int i = 0; i < kElemsPerThread; ++i)  // plain loads: the C2C may run in place
-      z[i] = live ? src[(size_t)i * xs * C] : make_float2(0.f, 0.f);
+      z[i] = live && (!PRUNED || kInv || x0 + i * xs < n) ? src[(size_t)i * xs * C] : make_float2(0.f, 0.f);
     first_pass_regs<kInv>(Z, z, x0);
   } else {  // C2R: rows k = 0 .. L/2 of two complex columns per slot
     const float2* in = static_cast<const float2*>(vin) + ob * in_outer;
@@ -127,7 +144,7 @@ __global__ void __launch_bounds__(1024) lateral_kernel(const void* vin, void* vo
 #pragma unroll
       for (int i = 0; i < kElemsPerThread; ++i) {
         const int x = x0 + i * xs;
-        out[(size_t)x * C + c0 + f] = Z[x];
+        if (!PRUNED || !kInv || x < n) out[(size_t)x * C + c0 + f] = Z[x];
       }
     }
   } else {
@@ -136,7 +153,17 @@ __global__ void __launch_bounds__(1024) lateral_kernel(const void* vin, void* vo
 #pragma unroll
       for (int i = 0; i < kElemsPerThread; ++i) {
         const int x = x0 + i * xs;
-        *reinterpret_cast<float2*>(out + (size_t)x * C + c0 + 2 * f) = Z[x];
+        if (!PRUNED) {
+          *reinterpret_cast<float2*>(out + (size_t)x * C + c0 + 2 * f) = Z[x];
+        } else if (x < n) {
+          float* o = out + (size_t)x * C + c0 + 2 * f;
+          if (pairs) {
+            *reinterpret_cast<float2*>(o) = Z[x];
+          } else {
+            o[0] = Z[x].x;
+            o[1] = Z[x].y;
+          }
+        }
       }
     }
   }
@@ -159,51 +186,64 @@ bool lateral_supported(int L, int C) {
   return lateral_smem_bytes(L) <= 200 * 1024;
 }
 
-template <int KIND, int FP>
+template <int KIND, int FP, bool PRUNED>
 static cudaError_t lat_launch(const void* in, void* out, int L, int C, int outer, long long in_outer,
-                              long long out_outer, const float2* tw, int twstride, cudaStream_t s) {
+                              long long out_outer, const float2* tw, int twstride, cudaStream_t s, int n) {
   const size_t smem = lateral_smem_bytes(L);
   cudaError_t e =
-      cudaFuncSetAttribute(lateral_kernel<KIND, FP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(lateral_kernel<KIND, FP, PRUNED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int mshift = 0;
   while ((1 << mshift) < L) ++mshift;
   const int threads = FP * (L / kElemsPerThread);
   constexpr int CPT = (KIND == kLatC2C || KIND == kLatC2CInv) ? FP : 2 * FP;
   dim3 grid((C + CPT - 1) / CPT, outer);
-  lateral_kernel<KIND, FP><<<grid, threads, smem, s>>>(in, out, L, mshift, C, in_outer, out_outer, tw, twstride);
+  const void* real = KIND == kLatR2C ? in : out;
+  const int pairs = (reinterpret_cast<uintptr_t>(real) & 7) == 0;
+  lateral_kernel<KIND, FP, PRUNED>
+      <<<grid, threads, smem, s>>>(in, out, L, mshift, C, in_outer, out_outer, tw, twstride, n, pairs);
   return cudaGetLastError();
 }
 
-template <int KIND>
-static cudaError_t lat_dispatch(const void* in, void* out, int L, int C, int outer, long long in_outer,
-                                long long out_outer, const float2* tw, int twstride, cudaStream_t s) {
+// in_full / out_full: outer strides for L (complex kinds) or L/2 + 1 points; the pruned side has n.
+template <int KIND, bool PRUNED>
+static cudaError_t lat_dispatch(const void* in, void* out, int L, int C, int outer, const float2* tw, int twstride,
+                                cudaStream_t s, int n) {
+  const long long full = (long long)L * C, half = (long long)(L / 2 + 1) * C, part = (long long)n * C;
+  const long long io = KIND == kLatC2R ? half : KIND == kLatC2CInv ? full : part;
+  const long long oo = KIND == kLatR2C ? half : KIND == kLatC2C ? full : part;
   switch (lateral_slots_per_cta(L)) {
-    case 8: return lat_launch<KIND, 8>(in, out, L, C, outer, in_outer, out_outer, tw, twstride, s);
-    case 4: return lat_launch<KIND, 4>(in, out, L, C, outer, in_outer, out_outer, tw, twstride, s);
-    case 2: return lat_launch<KIND, 2>(in, out, L, C, outer, in_outer, out_outer, tw, twstride, s);
-    default: return lat_launch<KIND, 1>(in, out, L, C, outer, in_outer, out_outer, tw, twstride, s);
+    case 8: return lat_launch<KIND, 8, PRUNED>(in, out, L, C, outer, io, oo, tw, twstride, s, n);
+    case 4: return lat_launch<KIND, 4, PRUNED>(in, out, L, C, outer, io, oo, tw, twstride, s, n);
+    case 2: return lat_launch<KIND, 2, PRUNED>(in, out, L, C, outer, io, oo, tw, twstride, s, n);
+    default: return lat_launch<KIND, 1, PRUNED>(in, out, L, C, outer, io, oo, tw, twstride, s, n);
   }
+}
+
+template <int KIND>
+static cudaError_t lat_any(const void* in, void* out, int L, int C, int outer, const float2* tw, int twstride,
+                           cudaStream_t s, int n) {
+  if (n > 0 && n < L) return lat_dispatch<KIND, true>(in, out, L, C, outer, tw, twstride, s, n);
+  return lat_dispatch<KIND, false>(in, out, L, C, outer, tw, twstride, s, L);
 }
 
 // out[o][k][c] = sum_x e^{-2 pi i k x / L} in[o][x][c], k = 0..L/2.
 cudaError_t launch_lateral_r2c(const float* in, float2* out, int L, int C, int outer, const float2* tw, int twstride,
-                               cudaStream_t s) {
-  return lat_dispatch<kLatR2C>(in, out, L, C, outer, (long long)L * C, (long long)(L / 2 + 1) * C, tw, twstride, s);
+                               cudaStream_t s, int n) {
+  return lat_any<kLatR2C>(in, out, L, C, outer, tw, twstride, s, n);
 }
 
 // out[o][x][c] = sum over the Hermitian extension of in[o][k][c] of e^{+2 pi i k x / L} (unnormalised C2R).
 cudaError_t launch_lateral_c2r(const float2* in, float* out, int L, int C, int outer, const float2* tw, int twstride,
-                               cudaStream_t s) {
-  return lat_dispatch<kLatC2R>(in, out, L, C, outer, (long long)(L / 2 + 1) * C, (long long)L * C, tw, twstride, s);
+                               cudaStream_t s, int n) {
+  return lat_any<kLatC2R>(in, out, L, C, outer, tw, twstride, s, n);
 }
 
-// out[o][k][c] = sum_x e^{-+2 pi i k x / L} in[o][x][c]; in place allowed (each CTA owns its columns).
+// out[o][k][c] = sum_x e^{-+2 pi i k x / L} in[o][x][c]; in place allowed when not pruned (each CTA owns its columns).
 cudaError_t launch_lateral_c2c(const float2* in, float2* out, int L, int C, int outer, bool inverse, const float2* tw,
-                               int twstride, cudaStream_t s) {
-  if (inverse)
-    return lat_dispatch<kLatC2CInv>(in, out, L, C, outer, (long long)L * C, (long long)L * C, tw, twstride, s);
-  return lat_dispatch<kLatC2C>(in, out, L, C, outer, (long long)L * C, (long long)L * C, tw, twstride, s);
+                               int twstride, cudaStream_t s, int n) {
+  if (inverse) return lat_any<kLatC2CInv>(in, out, L, C, outer, tw, twstride, s, n);
+  return lat_any<kLatC2C>(in, out, L, C, outer, tw, twstride, s, n);
 }
 
 // In-place FFT of contiguous lines (the depth transform of Eq. fft-1 and its
@@ -260,6 +300,57 @@ cudaError_t launch_rows_c2c(float2* data, int L, int rows, bool inverse, const f
     if (e != cudaSuccess) return e;
     rows_fft_kernel<false><<<ctas, threads, smem, s>>>(data, L, mshift, rows, tw, twstride);
   }
+  return cudaGetLastError();
+}
+
+// The depth stage of the forward model: lines of n image layers, zero-padded to
+// the box depth L and transformed; only c_j = F[j] + F[L - j] is wanted (each
+// node pair carries the sum), so a line costs n values read and L/2 + 1
+// written instead of L read and L written, and the padded box itself is never
+// in memory.
+__global__ void __launch_bounds__(1024) rows_fold_kernel(const float2* __restrict__ in, int n, float2* __restrict__ out,
+                                                         int L, int mshift, int rows, const float2* __restrict__ tw,
+                                                         int twstride) {
+  extern __shared__ float2 smem[];
+  const int tpr = L / kElemsPerThread;
+  const int slot = threadIdx.x / tpr;
+  const int lane = threadIdx.x - slot * tpr;
+  const int row = blockIdx.x * (blockDim.x / tpr) + slot;
+  const bool valid = row < rows;
+  float2* X = smem + slot * lateral_slot(L);
+  {
+    const float2* line = in + (size_t)(valid ? row : 0) * n;
+    float2 v[kElemsPerThread];
+#pragma unroll
+    for (int r = 0; r < kElemsPerThread; ++r) {
+      const int z = lane + r * tpr;
+      v[r] = z < n ? __ldg(line + z) : make_float2(0.f, 0.f);
+    }
+    first_pass_regs<false>(X, v, lane);
+  }
+  __syncthreads();
+  fft_rest<false, kLayoutFlat>(X, L, mshift, lane, tpr, tw, twstride);
+  if (!valid) return;
+  float2* o = out + (size_t)row * (L / 2 + 2);
+  for (int j = lane; j <= L / 2; j += tpr) {
+    float2 y = X[j];
+    if (j > 0 && j < L / 2) y = cadd(y, X[L - j]);
+    o[j] = y;
+  }
+}
+
+cudaError_t launch_rows_fold(const float2* in, int n, float2* out, int L, int rows, const float2* tw, int twstride,
+                             cudaStream_t s) {
+  if (L < 32 || (L & (L - 1)) != 0 || L / kElemsPerThread > 1024) return cudaErrorInvalidValue;
+  int mshift = 0;
+  while ((1 << mshift) < L) ++mshift;
+  const int tpr = L / kElemsPerThread;
+  const int threads = tpr > 128 ? tpr : 128;
+  const int rpc = threads / tpr;
+  const size_t smem = (size_t)rpc * lateral_slot(L) * sizeof(float2);
+  const cudaError_t e = cudaFuncSetAttribute(rows_fold_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  rows_fold_kernel<<<(rows + rpc - 1) / rpc, threads, smem, s>>>(in, n, out, L, mshift, rows, tw, twstride);
   return cudaGetLastError();
 }
 

@@ -155,6 +155,7 @@ void fill_row_scalars(const pai_geometry& g, int M, RowProblem& r) {
   r.M = M;
   r.nz = g.nz;
   r.lz = g.nz / 2 + 1;
+  r.zstride = g.nz;
   r.n1 = n1;
   r.n2 = n2;
   r.rows = n1 * (n2 / 2 + 1);

@@ -1029,10 +1029,11 @@ __device__ __forceinline__ bool adjoint_pairs(const RowProblem& P, const WindowP
   bool mirror = true;
   int np = 0;
   if (valid) {
-    const float2* Zs = P.fh + (size_t)row * P.nz;  // ZF: the row's depth spectrum Fbar[l mod nz]
+    const float2* Zs = P.fh + (size_t)row * P.zstride;  // ZF: the row's depth spectrum Fbar[l mod nz]
     if (ZF && P.qmode) {
       // forward model: pair j (j = 0..nz/2) carries c_j / 2 on both nodes,
-      // c_j = F[j] + F[-j] (F[0], F[nz/2] alone); wscale holds 1 / (2 n_lat nz)
+      // c_j = F[j] + F[-j] (F[0], F[nz/2] alone), stored by the depth stage at
+      // Zs[j]; wscale holds 1 / (2 n_lat nz)
       const float2 S = P.rowS[row];
       np = nzh + 1;
       for (int j = lane; j <= nzh; j += tpr) {
@@ -1040,8 +1041,7 @@ __device__ __forceinline__ bool adjoint_pairs(const RowProblem& P, const WindowP
         int j0;
         float fr, rx;
         node_position(S, zt, P.B2hi, P.B2lo, j0, fr, rx);
-        float2 y = Zs[j];
-        if (j > 0 && j < nzh) y = cadd(y, Zs[P.nz - j]);
+        const float2 y = Zs[j];
         const float2 pb = make_float2(P.wscale * y.x, P.wscale * y.y);
         const float2 ph = node_phase(j0, fr, nt, M, P.nt_over_M);
         const float2 qp = cmul(pb, ph), qn = cmul(pb, make_float2(ph.x, -ph.y));
@@ -1233,13 +1233,13 @@ __global__ void __launch_bounds__(1024) row_adjoint_kernel(RowLaunch L, WindowPo
     RowGeom rg;
     int nneg = 1, nn = 0;
     // ZF: the row's depth spectrum Fbar[l mod nz] (depth FFT of the lateral R2C of the image)
-    const float2* Zs = P.fh + (size_t)(valid ? row : 0) * P.nz;
+    const float2* Zs = P.fh + (size_t)(valid ? row : 0) * P.zstride;
     if (valid && ZF && P.qmode) {
       // Discrete forward model (the operator Q of Sec. 2 on a padded periodic
       // box): the row's temporal samples are sum_j c_j cos(2 pi nu_j n / nt)
       // over the depth frequencies j = 0..nz/2, nu_j >= 0 the frequency of
       // |K| (j = 0 included: its frequency is the lateral |K|), with
-      // c_j = F[j] + F[-j] (F[0], F[nz/2] alone).  Each cosine is the node pair
+      // c_j = F[j] + F[-j] (F[0], F[nz/2] alone; Zs[j]).  Each cosine is the node pair
       // +-nu_j with value c_j / 2 (wscale holds 1 / (2 n_lat nz)); the spread
       // below and the inverse FFT then sum the pairs like any adjoint row.
       rg.S = P.rowS[row];
@@ -1252,12 +1252,7 @@ __global__ void __launch_bounds__(1024) row_adjoint_kernel(RowLaunch L, WindowPo
         float frp, fr, rx;
         node_position(rg.S, zt, P.B2hi, P.B2lo, j0p, frp, rx);
         negate_node(j0p, frp, j0, fr);
-        float2 y = Zs[j];
-        if (j > 0 && j < nzh) {
-          const float2 y2 = Zs[P.nz - j];
-          y.x += y2.x;
-          y.y += y2.y;
-        }
+        const float2 y = Zs[j];
         const float2 pb = make_float2(P.wscale * y.x, P.wscale * y.y);
         const float2 qp = cmul(pb, node_phase(j0p, frp, nt, M, P.nt_over_M));
         const float2 qn = cmul(pb, node_phase(j0, fr, nt, M, P.nt_over_M));
