@@ -167,6 +167,19 @@ pai_status plan_malloc(pai_plan_s* P, void** ptr, size_t bytes) {
   return PAI_OK;
 }
 
+// Host-to-device upload and zeroing of a plan's buffers while it is built, in
+// the order of cap_stream, on which the tuner launches: that stream does not
+// wait for the legacy stream, where a plain cudaMemcpy from pageable memory may
+// still be on its way when the call returns (a kernel launched at once could
+// read the work items or tables of freed memory).  Returns when the copy is done.
+pai_status plan_upload(pai_plan_s* P, void* dst, const void* src, size_t bytes) {
+  const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, P->cap_stream);
+  return cuda_status(e != cudaSuccess ? e : cudaStreamSynchronize(P->cap_stream));
+}
+pai_status plan_zero(pai_plan_s* P, void* dst, size_t bytes) {
+  return cuda_status(cudaMemsetAsync(dst, 0, bytes, P->cap_stream));
+}
+
 // cuFFT plan creation of a plan; with PAI_FAULT_CUFFT_PLAN = n the n-th
 // creation (counted from 0 over the plan's build) reports a cuFFT failure
 // without calling cuFFT.
@@ -843,9 +856,9 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
   PAI_TRY(plan_malloc(P, (void**)&P->d_tw, tw.size() * sizeof(float2)));
   PAI_TRY(plan_malloc(P, (void**)&P->d_problems, count * sizeof(RowProblem)));
   PAI_TRY(plan_malloc(P, (void**)&P->d_counter, 4 * sizeof(int)));
-  PAI_CUDA(cudaMemset(P->d_counter, 0, 4 * sizeof(int)));
-  PAI_CUDA(cudaMemcpy(P->d_tables, tables.data(), tab_off * sizeof(float), cudaMemcpyHostToDevice));
-  PAI_CUDA(cudaMemcpy(P->d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice));
+  PAI_TRY(plan_zero(P, P->d_counter, 4 * sizeof(int)));
+  PAI_TRY(plan_upload(P, P->d_tables, tables.data(), tab_off * sizeof(float)));
+  PAI_TRY(plan_upload(P, P->d_tw, tw.data(), tw.size() * sizeof(float2)));
 
   std::vector<RowProblem> rp(count);
   for (int i = 0; i < count; ++i) {
@@ -941,8 +954,8 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     P->d_items_fwd = nullptr;
     P->items_fwd_bytes = items.size() * sizeof(WorkItem);
     PAI_TRY(plan_malloc(P, (void**)&P->d_items_fwd, P->items_fwd_bytes));
-    PAI_CUDA(cudaMemcpy(P->d_items_fwd, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
-    PAI_CUDA(cudaMemcpy(P->d_problems, rp.data(), count * sizeof(RowProblem), cudaMemcpyHostToDevice));
+    PAI_TRY(plan_upload(P, P->d_items_fwd, items.data(), items.size() * sizeof(WorkItem)));
+    PAI_TRY(plan_upload(P, P->d_problems, rp.data(), count * sizeof(RowProblem)));
     return PAI_OK;
   };
   // CTA shape of the adjoint row kernel (row slots, then the node lists)
@@ -1013,7 +1026,7 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     P->d_items_adj = nullptr;
     P->items_adj_bytes = items.size() * sizeof(WorkItem);
     PAI_TRY(plan_malloc(P, (void**)&P->d_items_adj, P->items_adj_bytes));
-    PAI_CUDA(cudaMemcpy(P->d_items_adj, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
+    PAI_TRY(plan_upload(P, P->d_items_adj, items.data(), items.size() * sizeof(WorkItem)));
     return PAI_OK;
   };
   const char* env_tune = std::getenv("PAI_AUTOTUNE");
@@ -1047,7 +1060,7 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
         fill_row_tables(p.g, p.c_eff, p.H, p.beta, &tables_c[p.pre_off], &tables_c[p.rowS_off], &tables_c[p.zt_off]);
         fill_row_scalars(p.g, p.M, rp[i]);
       }
-      PAI_CUDA(cudaMemcpy(P->d_tables, tables_c.data(), tab_off * sizeof(float), cudaMemcpyHostToDevice));
+      PAI_TRY(plan_upload(P, P->d_tables, tables_c.data(), tab_off * sizeof(float)));
       tpr_max = P->Mmax / kElemsPerThread;
       return PAI_OK;
   };
@@ -1062,7 +1075,7 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     cudaEvent_t e0, e1;
     PAI_CUDA(cudaEventCreate(&e0));
     PAI_CUDA(cudaEventCreate(&e1));
-    PAI_CUDA(cudaMemset(P->d_pt, 0, pt_off * sizeof(float2)));
+    PAI_TRY(plan_zero(P, P->d_pt, pt_off * sizeof(float2)));
     int best_i = -1;
     float best_ms = 1e30f;
     for (size_t k = 0; k < cands.size(); ++k) {
@@ -1115,7 +1128,7 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     cudaEvent_t e0, e1;
     PAI_CUDA(cudaEventCreate(&e0));
     PAI_CUDA(cudaEventCreate(&e1));
-    PAI_CUDA(cudaMemset(P->d_pt, 0, pt_off * sizeof(float2)));
+    PAI_TRY(plan_zero(P, P->d_pt, pt_off * sizeof(float2)));
     for (int T : {32, 64, 128, 256, 512, 1024}) {
       if (T < tpr_max) continue;
       if (finish_shape(T) != PAI_OK) continue;
@@ -1155,7 +1168,7 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     cudaEvent_t e0, e1;
     PAI_CUDA(cudaEventCreate(&e0));
     PAI_CUDA(cudaEventCreate(&e1));
-    PAI_CUDA(cudaMemset(P->d_fh, 0, fh_off * sizeof(float2)));
+    PAI_TRY(plan_zero(P, P->d_fh, fh_off * sizeof(float2)));
     for (int T : {32, 64, 128, 256, 512, 1024}) {
       if (T < tpr_max) continue;
       if (finish_shape_adj(T) != PAI_OK) continue;
@@ -1206,7 +1219,7 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     cudaEvent_t e0, e1;
     PAI_CUDA(cudaEventCreate(&e0));
     PAI_CUDA(cudaEventCreate(&e1));
-    PAI_CUDA(cudaMemset(P->d_fh, 0, fh_off * sizeof(float2)));
+    PAI_TRY(plan_zero(P, P->d_fh, fh_off * sizeof(float2)));
     float best_ms[5] = {1e30f, 1e30f, 1e30f, 1e30f, 1e30f};
     for (int mode = 0; mode < 5; ++mode) {
       if (mode == 3 && !P->pairs_ok) continue;
@@ -1251,8 +1264,8 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     float ms_zf = 1e30f, ms_cufft = 1e30f;
     if (cudaMalloc(&d_in, P->data_total * sizeof(float)) == cudaSuccess &&
         cudaMalloc(&d_out, P->img_total * sizeof(float)) == cudaSuccess &&
-        cudaMemset(d_in, 0, P->data_total * sizeof(float)) == cudaSuccess &&
-        cudaMemset(d_out, 0, P->img_total * sizeof(float)) == cudaSuccess) {
+        cudaMemsetAsync(d_in, 0, P->data_total * sizeof(float), P->cap_stream) == cudaSuccess &&
+        cudaMemsetAsync(d_out, 0, P->img_total * sizeof(float), P->cap_stream) == cudaSuccess) {
       cudaEvent_t e0, e1;
       cudaEventCreate(&e0);
       cudaEventCreate(&e1);
@@ -1735,7 +1748,7 @@ pai_status pai_set_cutoff(pai_plan_t plan, double eps) {
     std::vector<float> wf(w.begin(), w.end());
     float* d = nullptr;
     st = plan_malloc(plan, (void**)&d, wf.size() * sizeof(float));
-    if (st == PAI_OK) st = cuda_status(cudaMemcpy(d, wf.data(), wf.size() * sizeof(float), cudaMemcpyHostToDevice));
+    if (st == PAI_OK) st = plan_upload(plan, d, wf.data(), wf.size() * sizeof(float));
     if (st == PAI_OK) {
       plan->d_cut = d;
       plan->cut_R = cutoff_radius(eps);
