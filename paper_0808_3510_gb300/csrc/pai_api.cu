@@ -41,7 +41,7 @@ struct ProblemHost {
   int n1 = 0, n2 = 0, rows = 0, lz = 0, tpr = 0, rpc = 0;
   size_t data_off = 0, img_off = 0;   // floats into the concatenated data / image
   size_t pt_off = 0, fh_off = 0;      // complex values into the workspaces
-  size_t pre_off = 0, rowS_off = 0, zt_off = 0;
+  size_t pre_off = 0, rowS_off = 0, zt_off = 0, model_off = 0;
   cufftHandle lat_r2c = 0, lat_c2r = 0, img_c2r = 0, img_r2c = 0;
   bool made[4] = {false, false, false, false};  // which of the four handles cufftCreate made
   bool have_plans = false;
@@ -76,8 +76,12 @@ struct pai_plan_s {
   bool pairs_ok = false;                            // spread mode 3 applies to every problem of the plan
   size_t smem_adj3 = 0;                             // mode 3: shared memory of the adjoint row kernel
   int ctas_adj3 = 0;                                //         and its CTA count
-  bool pairs_atom_ok = false;                       // spread mode 4 applies to every problem of the plan
-  int ctas_adj4 = 0;                                // mode 4: CTA count (shared memory as mode 3)
+  // forward-model row kernel (spread mode 4): CTA shape, work items (units of one row, or two in 3-D)
+  bool model_ok = false;
+  int threads_model = 0, ctas_model = 0, nitems_model = 0;
+  size_t smem_model = 0;
+  WorkItem* d_items_model = nullptr;
+  size_t items_model_bytes = 0;
   bool any_paired = false;  // some problem's lateral spectrum is in the paired layout (RowProblem::paired)
   bool zf = false;      // forward: every stage by the library's kernels (depth-row layout)
   bool zf_adj = false;  // adjoint: the same choice, tuned separately
@@ -312,6 +316,7 @@ void release(pai_plan_s* P) {
   if (P->d_items_adj == P->d_items_fwd) P->d_items_adj = nullptr;
   cudaFree(P->d_items_fwd);
   cudaFree(P->d_items_adj);
+  cudaFree(P->d_items_model);
   cudaFree(P->d_counter);
   cudaFree(P->d_cufft_work);
   for (void* w : P->branch_work) cudaFree(w);
@@ -350,6 +355,11 @@ RowLaunch make_launch(pai_plan_s* P, bool adjoint) {
   L.bin_offset = P->bin_offset;
   L.bin_slot = P->bin_slot;
   L.spread_mode = P->spread_mode;
+  if (adjoint && P->spread_mode == 4) {
+    L.items = P->d_items_model;
+    L.nitems = P->nitems_model;
+    L.model_pair = P->probs[0].g.dim == 3 ? 1 : 0;
+  }
   L.paired = !adjoint && P->any_paired ? 1 : 0;
   return L;
 }
@@ -357,10 +367,14 @@ RowLaunch make_launch(pai_plan_s* P, bool adjoint) {
 pai_status enqueue_row(pai_plan_s* P, bool adjoint, cudaStream_t s, int threads, int ctas, size_t smem,
                        bool zf = false) {
   RowLaunch L = make_launch(P, adjoint);
-  if (adjoint && (P->spread_mode == 3 || P->spread_mode == 4)) {
-    // the pair-spread kernels' own occupancy gives their CTA counts
+  if (adjoint && P->spread_mode == 3) {
+    // the pair-spread kernel has its own shared memory and occupancy
     smem = P->smem_adj3;
-    ctas = P->spread_mode == 3 ? P->ctas_adj3 : P->ctas_adj4;
+    ctas = P->ctas_adj3;
+  } else if (adjoint && P->spread_mode == 4) {
+    threads = P->threads_model;
+    smem = P->smem_model;
+    ctas = P->ctas_model;
   }
   cudaError_t e = adjoint ? launch_row_adjoint(L, P->poly, threads, ctas, smem, s, zf)
                           : launch_row_forward(L, P->poly, threads, ctas, smem, s, zf);
@@ -819,6 +833,8 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     tab_off = align4(tab_off + 2 * (size_t)p.rows);
     p.zt_off = tab_off;
     tab_off = align4(tab_off + 4 * (size_t)p.lz);
+    p.model_off = tab_off;
+    if (qmode) tab_off = align4(tab_off + 2 * (size_t)p.g.nt);
     P->rows_total += p.rows;
     const int half = p.n2 / 2;
     long long mirror_rows = (long long)p.n1 * std::max(0, half - 1);
@@ -832,6 +848,8 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
   std::vector<float> tables(tab_off, 0.0f);
   for (auto& p : P->probs)
     fill_row_tables(p.g, p.c_eff, p.H, p.beta, &tables[p.pre_off], &tables[p.rowS_off], &tables[p.zt_off]);
+  if (qmode)
+    for (auto& p : P->probs) fill_model_table(p.g, p.M, p.c_eff, p.H, p.beta, &tables[p.model_off]);
   P->TW = tw_need;  // covers every window candidate's padded length
   for (auto& p : P->probs) {
     p.own_lateral = p.g.dim == 2 && lateral_supported(p.g.nx, p.g.nt);
@@ -869,11 +887,12 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     r.prescale = P->d_tables + p.pre_off;
     r.rowS = reinterpret_cast<const float2*>(P->d_tables + p.rowS_off);
     r.zt = reinterpret_cast<const float4*>(P->d_tables + p.zt_off);
-    fill_row_scalars(p.g, p.M, r);
+    fill_row_scalars(p.g, p.M, p.H, r);
     r.paired = p.paired ? 1 : 0;
     if (qmode) {
       r.qmode = 1;
       r.zstride = p.g.nz / 2 + 2;
+      r.model_tab = reinterpret_cast<const float2*>(P->d_tables + p.model_off);
       r.wscale = (float)(0.5 / ((double)r.n1 * r.n2 * p.g.nz));
     }
   }
@@ -987,39 +1006,25 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     if (P->smem_adj > (size_t)smem_optin) return PAI_ERR_UNSUPPORTED;
     const int occ_a = row_kernel_max_ctas_per_sm(1, T, P->smem_adj, P->H, P->zf);
     if (occ_a < 1) return PAI_ERR_UNSUPPORTED;
-    // spread mode 3 (node pairs spread by one warp per row): windowed
-    // methods, rows of one or two warps, and 32 consecutive pairs spanning
-    // fewer than M - 2H cells (consecutive nodes of one sign are at most
-    // M c dt / (nz dz) cells apart)
-    // spread mode 4 (every warp of the row, atomics): windowed methods and
-    // rows of whole warps
-    P->pairs_ok = !method_interp(P->method) && std::getenv("PAI_NO_PAIRS") == nullptr;
-    P->pairs_atom_ok = P->pairs_ok;
-    for (auto& p : P->probs) {
-      const double g1 = std::ceil((double)p.M * p.g.c * p.g.dt / (p.g.nz * p.g.dz)) + 1.0;
-      if (p.tpr != 32 && p.tpr != 64) P->pairs_ok = false;
-      if (!(32.0 * g1 + 2.0 * P->H + 2.0 < (double)p.M)) P->pairs_ok = false;
-      if (p.tpr % 32 != 0) P->pairs_atom_ok = false;
-    }
-    P->smem_adj3 = P->smem_adj;
+    // spread mode 3 (node pairs into band grids): windowed methods, as long as
+    // the bands fit in shared memory (up to c dt / dz = 3.4 at M = 8192, 1.7 at
+    // 16384, far more for shorter rows)
+    P->pairs_ok = !qmode && !method_interp(P->method) && std::getenv("PAI_NO_PAIRS") == nullptr;
+    P->smem_adj3 = 0;
+    for (int i = 0; i < count; ++i)
+      P->smem_adj3 = std::max(P->smem_adj3, (size_t)(T / P->probs[i].tpr) * (size_t)rp[i].band_slot * sizeof(float2));
+    if (P->smem_adj3 > (size_t)smem_optin) P->pairs_ok = false;
     P->ctas_adj3 = 0;
-    P->ctas_adj4 = 0;
     if (P->pairs_ok) {
       const int occ3 = row_kernel_max_ctas_per_sm(2, T, P->smem_adj3, P->H, P->zf);
       if (occ3 < 1) P->pairs_ok = false;
       P->ctas_adj3 = occ3 * sms;
-    }
-    if (P->pairs_atom_ok) {
-      const int occ4 = row_kernel_max_ctas_per_sm(4, T, P->smem_adj3, P->H, P->zf);
-      if (occ4 < 1) P->pairs_atom_ok = false;
-      P->ctas_adj4 = occ4 * sms;
     }
     std::vector<WorkItem> items;
     build_items(T, items);
     P->nitems_adj = (int)items.size();
     P->ctas_adj = std::min(P->nitems_adj, occ_a * sms);
     P->ctas_adj3 = std::min(P->nitems_adj, P->ctas_adj3);
-    P->ctas_adj4 = std::min(P->nitems_adj, P->ctas_adj4);
     if (P->d_items_adj == P->d_items_fwd) P->d_items_adj = nullptr;
     if (P->d_items_adj) P->alloc_used -= (long long)P->items_adj_bytes;
     cudaFree(P->d_items_adj);
@@ -1027,6 +1032,30 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     P->items_adj_bytes = items.size() * sizeof(WorkItem);
     PAI_TRY(plan_malloc(P, (void**)&P->d_items_adj, P->items_adj_bytes));
     PAI_TRY(plan_upload(P, P->d_items_adj, items.data(), items.size() * sizeof(WorkItem)));
+    return PAI_OK;
+  };
+  // CTA shape of the forward-model row kernel (one problem: the box)
+  auto finish_shape_model = [&](int T) -> pai_status {
+    const ProblemHost& p = P->probs[0];
+    const bool pair = p.g.dim == 3;
+    const int tpu = pair ? 2 * p.tpr : p.tpr, upc = T / tpu;
+    const int units = pair ? (p.n1 / 2 + 1) * (p.n2 / 2 + 1) : p.rows;
+    if (upc < 1 || T > 1024) return PAI_ERR_UNSUPPORTED;
+    P->threads_model = T;
+    P->smem_model = (size_t)upc * (size_t)rp[0].model_slot * sizeof(float2);
+    if (P->smem_model > (size_t)smem_optin) return PAI_ERR_UNSUPPORTED;
+    const int occ = row_kernel_max_ctas_per_sm(pair ? 5 : 4, T, P->smem_model, P->H, true);
+    if (occ < 1) return PAI_ERR_UNSUPPORTED;
+    std::vector<WorkItem> items;
+    for (int u = 0; u < units; u += upc) items.push_back(WorkItem{0, u});
+    P->nitems_model = (int)items.size();
+    P->ctas_model = std::min(P->nitems_model, occ * sms);
+    if (P->d_items_model) P->alloc_used -= (long long)P->items_model_bytes;
+    cudaFree(P->d_items_model);
+    P->d_items_model = nullptr;
+    P->items_model_bytes = items.size() * sizeof(WorkItem);
+    PAI_TRY(plan_malloc(P, (void**)&P->d_items_model, P->items_model_bytes));
+    PAI_TRY(plan_upload(P, P->d_items_model, items.data(), P->items_model_bytes));
     return PAI_OK;
   };
   const char* env_tune = std::getenv("PAI_AUTOTUNE");
@@ -1058,7 +1087,7 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
         ProblemHost& p = P->probs[i];
         p.tpr = p.M / kElemsPerThread;
         fill_row_tables(p.g, p.c_eff, p.H, p.beta, &tables_c[p.pre_off], &tables_c[p.rowS_off], &tables_c[p.zt_off]);
-        fill_row_scalars(p.g, p.M, rp[i]);
+        fill_row_scalars(p.g, p.M, p.H, rp[i]);
       }
       PAI_TRY(plan_upload(P, P->d_tables, tables_c.data(), tab_off * sizeof(float)));
       tpr_max = P->Mmax / kElemsPerThread;
@@ -1172,6 +1201,7 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     for (int T : {32, 64, 128, 256, 512, 1024}) {
       if (T < tpr_max) continue;
       if (finish_shape_adj(T) != PAI_OK) continue;
+      P->spread_mode = P->pairs_ok ? 3 : 1;  // the spread that will most likely be kept
       float best = 1e30f;
       for (int rep = 0; rep < 4; ++rep) {
         cudaEventRecord(e0, P->cap_stream);
@@ -1205,25 +1235,57 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
                  : std::strcmp(env_spread, "runs") == 0 ? 2
                  : std::strcmp(env_spread, "pairs") == 0 ? 3
                  : std::strcmp(env_spread, "pairs_atomic") == 0 ? 4 : -1;
-  if (env_mode == 3 && !P->pairs_ok) env_mode = 0;
-  if (env_mode == 4 && !P->pairs_atom_ok) env_mode = 1;
-  P->spread_det = P->pairs_ok ? 3 : 0;
+  // (the band grids took the place of both pair spreads)
+  if (env_mode == 4) env_mode = P->pairs_ok || qmode ? 3 : 1;
+  if (env_mode == 3 && !P->pairs_ok && !qmode) env_mode = 0;
+  // forward models run their own row kernel (see row_model_kernel) unless it
+  // does not fit or one of the list spreads is forced; its CTA size is timed
+  if (qmode && (env_mode < 0 || env_mode == 3)) {
+    const int tpu = (P->probs[0].g.dim == 3 ? 2 : 1) * P->probs[0].tpr;
+    int best_T = 0;
+    float best_ms = 1e30f;
+    cudaEvent_t e0, e1;
+    PAI_CUDA(cudaEventCreate(&e0));
+    PAI_CUDA(cudaEventCreate(&e1));
+    PAI_TRY(plan_zero(P, P->d_fh, fh_off * sizeof(float2)));
+    P->spread_mode = 4;
+    for (int T : {32, 64, 128, 256, 512, 1024}) {
+      if (T < tpu || finish_shape_model(T) != PAI_OK) continue;
+      float best = 1e30f;
+      for (int rep = 0; rep < 3; ++rep) {
+        cudaEventRecord(e0, P->cap_stream);
+        if (enqueue_row(P, true, P->cap_stream, T, 0, 0, true) != PAI_OK) break;
+        cudaEventRecord(e1, P->cap_stream);
+        cudaEventSynchronize(e1);
+        float ms = 0;
+        cudaEventElapsedTime(&ms, e0, e1);
+        if (rep > 0) best = std::min(best, ms);
+      }
+      std::snprintf(logline, sizeof logline, "forward model CTA: %d threads: row kernel %.4f ms\n", T, best);
+      P->tune_log += logline;
+      if (best < best_ms) { best_ms = best; best_T = T; }
+    }
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
+    cudaGetLastError();
+    P->model_ok = best_T > 0 && finish_shape_model(best_T) == PAI_OK;
+    env_mode = P->model_ok ? 4 : -1;
+  }
+  P->spread_det = P->model_ok ? 4 : P->pairs_ok ? 3 : 0;
   if (env_mode >= 0) {
     P->spread_tuned = env_mode;
   } else if (have_wis) {
-    P->spread_tuned = wis.spread_tuned == 3 && !P->pairs_ok         ? 0
-                      : wis.spread_tuned == 4 && !P->pairs_atom_ok ? 1
-                                                                   : wis.spread_tuned;
+    P->spread_tuned = wis.spread_tuned == 3 && !P->pairs_ok ? 0 : wis.spread_tuned;
     P->spread_det = wis.spread_det == 3 && !P->pairs_ok ? 0 : wis.spread_det;
   } else if (tune || qmode) {
     cudaEvent_t e0, e1;
     PAI_CUDA(cudaEventCreate(&e0));
     PAI_CUDA(cudaEventCreate(&e1));
     PAI_TRY(plan_zero(P, P->d_fh, fh_off * sizeof(float2)));
-    float best_ms[5] = {1e30f, 1e30f, 1e30f, 1e30f, 1e30f};
-    for (int mode = 0; mode < 5; ++mode) {
+    P->spread_mode = 0;
+    float best_ms[4] = {1e30f, 1e30f, 1e30f, 1e30f};
+    for (int mode = 0; mode < 4; ++mode) {
       if (mode == 3 && !P->pairs_ok) continue;
-      if (mode == 4 && !P->pairs_atom_ok) continue;
       P->spread_mode = mode;
       for (int rep = 0; rep < 4; ++rep) {
         cudaEventRecord(e0, P->cap_stream);
@@ -1238,16 +1300,15 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cudaGetLastError();
-    static const char* kSpreadName[5] = {"tap phases", "atomics per node", "atomics per run", "node pairs",
-                                         "node pairs, atomics"};
-    for (int mode = 0; mode < 5; ++mode)
+    static const char* kSpreadName[4] = {"tap phases", "atomics per node", "atomics per run", "node pairs"};
+    for (int mode = 0; mode < 4; ++mode)
       if (best_ms[mode] < 1e29f) {
         std::snprintf(logline, sizeof logline, "adjoint spread: %s: adjoint row kernel %.4f ms\n", kSpreadName[mode],
                       best_ms[mode]);
         P->tune_log += logline;
       }
     P->spread_tuned = 0;
-    for (int mode = 1; mode < 5; ++mode)
+    for (int mode = 1; mode < 4; ++mode)
       if (best_ms[mode] < best_ms[P->spread_tuned]) P->spread_tuned = mode;
     P->spread_det = (P->pairs_ok && best_ms[3] < best_ms[0]) ? 3 : 0;
   }
@@ -1561,7 +1622,7 @@ pai_status pai_profile_stages(pai_plan_t plan, const float* d_in, float* d_out, 
 
 pai_status pai_set_deterministic(pai_plan_t plan, int deterministic) {
   if (!plan || (deterministic != 0 && deterministic != 1)) return PAI_ERR_INVALID_ARG;
-  const int mode = deterministic ? (plan->spread_tuned == 3 ? 3 : plan->spread_det) : plan->spread_tuned;
+  const int mode = deterministic && plan->spread_tuned < 3 ? plan->spread_det : plan->spread_tuned;
   if (mode == plan->spread_mode) return PAI_OK;
   int prev = 0;
   cudaGetDevice(&prev);

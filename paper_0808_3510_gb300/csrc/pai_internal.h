@@ -71,6 +71,9 @@ struct RowProblem {
   int qmode;               // adjoint kernel evaluates the discrete forward model (depth-row layout only)
   int zstride;             // depth-row layout: complex values from one row to the next (nz; in qmode
                            // the rows hold c_j, j = 0..nz/2, nz/2 + 2 values apart)
+  int band_ps, band_slot;  // adjoint pair spread: cells per phase of the band grid, complex values per row slot
+  int model_ps, model_slot;  // the same for the forward-model row kernel (per unit of one or two rows)
+  const float2* model_tab;   // forward-model row kernel: [nt] prescale times e^{-i pi n / (2M)}
   int paired;              // 2-D, forward: pt holds Z[k][m] (k < nx = n2, m < nt/2, row stride nt/2), the
                            // lateral DFT of the sample pairs p[x][2m] + i p[x][2m+1]; the forward row kernel
                            // separates row k's samples from Z[k] and Z[nx - k]
@@ -96,9 +99,9 @@ struct RowLaunch {
   int bin_slot;                // bytes of bins per row slot: chunk * (2H+1) complex, 16-aligned
   int spread_mode;             // adjoint spread: 0 tap phases (deterministic), 1 shared-memory atomics per
                                // node, 2 shared-memory atomics per run of nodes with equal j0, 3 node pairs
-                               // spread by one warp per row (deterministic; windowed methods, 32 or 64
-                               // threads per row), 4 node pairs spread by every warp of the row with
-                               // shared-memory atomics (windowed methods, a multiple of 32 threads per row)
+                               // into band grids (deterministic; windowed methods; not qmode), 4 the
+                               // forward-model row kernel (deterministic; qmode only)
+  int model_pair;              // spread mode 4: units of two rows (3-D)
   int paired;                  // forward: some problem is in the paired layout (RowProblem::paired)
 };
 
@@ -153,7 +156,12 @@ void fill_row_tables(const pai_geometry& g, double c_eff, int H, double beta, fl
 inline int method_window(int method) { return method == PAI_METHOD_TSINC ? 1 : 0; }
 inline bool method_interp(int method) { return method == PAI_METHOD_LINEAR || method == PAI_METHOD_NEAREST; }
 // Scalar fields of RowProblem (everything except pointers and rpc).
-void fill_row_scalars(const pai_geometry& g, int M, RowProblem& r);
+void fill_row_scalars(const pai_geometry& g, int M, int H, RowProblem& r);
+// Cells per phase of a band grid for `cells` cells of 2^shift bytes, and the complex values a slot of `warps` warps
+// needs for the band, its spills and bounds, at least `fft` of them.
+void band_layout(double cells, int H, int shift, int warps, long long fft, int& ps, int& slot);
+// model_tab of RowProblem: [2 nt] floats.
+void fill_model_table(const pai_geometry& g, int M, double c_eff, int H, double beta, float* tab);
 // Two-level twiddle table for transforms of every length dividing TW (a power
 // of two): tw[j] = w^j for j < kTwLo, tw[kTwLo + i] = w^(kTwLo i) for
 // i < TW / kTwLo, w = e^{-2 pi i / TW}; w^k = tw[kTwLo + (k >> 6)] tw[k & 63].
@@ -188,7 +196,7 @@ cudaError_t launch_rows_c2c(float2* data, int L, int rows, bool inverse, const f
 cudaError_t launch_rows_fold(const float2* in, int n, float2* out, int L, int rows, const float2* tw, int twstride,
                              cudaStream_t s);
 // kind: 0 forward row kernel, 1 adjoint row kernel, 2 adjoint row kernel with the pair spread, 3 forward row
-// kernel for launches with problems in the paired layout, 4 adjoint with the atomic pair spread
+// kernel for launches with problems in the paired layout, 4 forward-model row kernel, 5 the same in units of two rows
 int row_kernel_max_ctas_per_sm(int kind, int threads, size_t smem, int H, bool zf = false);
 
 // Data cutoff w_cut (pai_cutoff.cu).  R = ceil(sqrt(eps)); the table holds

@@ -26,17 +26,6 @@ __host__ __device__ inline int lateral_slot(int L) { return L + (L >> 5) + 4; }
 
 enum : int { kLatR2C = 0, kLatC2R = 1, kLatC2C = 2, kLatC2CInv = 3 };
 
-// The values a thread loads, column elements x0 + i L/16 (i = 0..15), are the
-// inputs of butterfly x0 of the first radix-16 Stockham pass (Ns = 1): that
-// pass runs on them in registers and writes its outputs 16 x0 + r in the
-// padded layout, ready for fft_rest.
-template <bool INV>
-__device__ __forceinline__ void first_pass_regs(float2* Z, float2 (&z)[kElemsPerThread], int x0) {
-  dft_reg<kElemsPerThread, INV>(z);
-#pragma unroll
-  for (int r = 0; r < kElemsPerThread; ++r) Z[PADI(x0 * kElemsPerThread + r)] = z[r];
-}
-
 // Two adjacent floats, one load when they start on an 8-byte boundary (pairs).
 template <bool CHECK>
 __device__ __forceinline__ float2 ldg_pair(const float2* p, int pairs) {

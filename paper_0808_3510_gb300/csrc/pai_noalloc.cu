@@ -69,7 +69,7 @@ extern "C" pai_status pai_spectrum_rows_noalloc(const pai_geometry* g_in, const 
   const int rpc = threads / tpr;
 
   RowProblem rp{};
-  fill_row_scalars(g, pp.M, rp);
+  fill_row_scalars(g, pp.M, pp.H, rp);
   rp.rpc = rpc;
   const int rows = rp.rows;
   const int nitems = (rows + rpc - 1) / rpc;

@@ -147,7 +147,30 @@ void fill_row_tables(const pai_geometry& g, double c_eff, int H, double beta, fl
   }
 }
 
-void fill_row_scalars(const pai_geometry& g, int M, RowProblem& r) {
+void band_layout(double cells, int H, int shift, int warps, long long fft, int& ps, int& slot) {
+  // 2H window cells and a few to spare; the phases start 2 (mod 8) 16-byte or 4 (mod 16) 8-byte cells apart, so that
+  // neighbouring nodes one, two or four cells apart fall on distinct banks
+  const int n = (int)std::min(1e7, std::ceil(cells)) + 2 * H + 8;
+  const int period = 128 >> shift, off = period / 4;
+  ps = (n + 3) / 4;
+  ps += ((off - ps % period) + period) % period;
+  const long long bytes = ((4LL * ps + (warps > 1 ? warps * (2 * H + 4) : 0)) << shift) + 8LL * warps;
+  const long long need = std::max(fft, (bytes + 7) / 8);
+  slot = (int)std::min<long long>(1 << 28, (need + 1) & ~1LL);
+}
+
+void fill_model_table(const pai_geometry& g, int M, double c_eff, int H, double beta, float* tab) {
+  // the prescale over (-nt, nt), theta_n = pi n / nt: the upper half of the table of 2 nt samples
+  std::vector<float> s(2 * (size_t)g.nt);
+  prescale_table(method_window(g.method), 2 * g.nt, c_eff, H, beta, 1.0, s.data());
+  for (int n = 0; n < g.nt; ++n) {
+    const double a = kPi * n / (2.0 * M), w = s[g.nt + n];
+    tab[2 * n] = (float)(w * std::cos(a));
+    tab[2 * n + 1] = (float)(-w * std::sin(a));
+  }
+}
+
+void fill_row_scalars(const pai_geometry& g, int M, int H, RowProblem& r) {
   int n1, n2;
   double d1, d2;
   lateral_axes(g, n1, n2, d1, d2);
@@ -171,6 +194,14 @@ void fill_row_scalars(const pai_geometry& g, int M, RowProblem& r) {
   r.wscale = (float)(2.0 * g.c * g.dt / g.dz * B / ((double)n1 * n2 * g.nz));
   r.nt_over_M = (float)((double)g.nt / M);
   r.method = g.method;
+  // band grid: the nodes of a row span at most B kz_max cells (the row K_lat = 0); on the forward model's doubled
+  // interval twice as many
+  const int warps = r.tpr > 32 ? r.tpr / 32 : 1;
+  band_layout(B * 0.5 / g.dz, H, 4, warps, r.slot, r.band_ps, r.band_slot);
+  const bool pair = g.dim == 3;
+  const int tpu = pair ? 2 * r.tpr : r.tpr;
+  band_layout(2 * B * 0.5 / g.dz, H, pair ? 4 : 3, tpu > 32 ? tpu / 32 : 1, (pair ? 2LL : 1LL) * r.slot, r.model_ps,
+              r.model_slot);
 }
 
 void twiddle_table(int TW, float2* tw) {

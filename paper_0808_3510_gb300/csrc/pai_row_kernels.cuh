@@ -483,6 +483,17 @@ __device__ __forceinline__ bool first_pass32(int M, int mshift, int nt) {
   return M == 2 * nt && mshift >= 9 && ((mshift - 5) & 3) == 0;
 }
 
+// The values a thread loads, elements x0 + i M/16 (i = 0..15), are the inputs
+// of butterfly x0 of the first radix-16 Stockham pass (Ns = 1): that pass runs
+// on them in registers and writes its outputs 16 x0 + r in the padded layout,
+// ready for fft_rest.
+template <bool INV>
+__device__ __forceinline__ void first_pass_regs(float2* Z, float2 (&z)[kElemsPerThread], int x0) {
+  dft_reg<kElemsPerThread, INV>(z);
+#pragma unroll
+  for (int r = 0; r < kElemsPerThread; ++r) Z[PADI(x0 * kElemsPerThread + r)] = z[r];
+}
+
 // Remaining passes after a first pass of radix 2^ns_shift (16 or 32: Ns on
 // entry); the last pass writes layout OUT.
 template <bool INV, int OUT, int CHAIN_R = 2>
@@ -504,35 +515,166 @@ __device__ __forceinline__ void fft_rest(float2* X, int M, int mshift, int lane,
   else if (rem == 1) fft_pass<2, INV, OUT, CHAIN_R>(X, M, Ns, lane, tpr, tw, twstride, active);
 }
 
-// Inverse length-M transform of an adjoint row with the crop fused: the
-// passes run remainder radix first and radix 16 last, and the last pass
-// (Ns = M/16, butterfly j = lane, outputs at positions m = j + r M/16) writes
-// the outputs that hold samples n = (m + nt/2) mod M < nt, times
-// s_n = scale * prescale[n], straight to dst[n].  At oversampling 2
+// 16-byte shared-memory accesses by 32-bit address (the band grid below).
+__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ float4 lds4(unsigned a) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(a)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 lds2(unsigned a) {
+  float2 v;
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void sts2(unsigned a, float2 v) {
+  asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void sts4(unsigned a, float4 v) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+
+// The band grid of an adjoint row (written by the pair spread, see
+// adjoint_band): cell c, counted from the row's first cell `lo`, holds the
+// sums P[c] over the +x nodes (first half of its 16 bytes) and N[c] over the
+// -x nodes (second half); the N sums belong to grid cell -c.  The oversampled
+// grid is U[m] = sum over c = m (mod M) of P[c] + sum over c = -m (mod M) of
+// N[c].  Cells are stored in four phases, cell c at (c mod 4) ps + c / 4.
+struct Band {
+  unsigned grid;  // shared-memory address of cell 0
+  int ps;         // cells per phase
+  int lo, n;      // first cell and number of cells in use
+};
+
+// First inverse pass (radix 16, Ns = 1) fed from the band grid (at most M cells
+// here), which shares the row slot's memory with the pass's output X: every
+// thread holds its 16 inputs before any writes.
+__device__ __forceinline__ void fft_first_pass_band(float2* X, int M, int lane, int tpr, const Band& b) {
+  constexpr int R = 16;
+  float2 v[R];
+  const int mask = M - 1;
+  const int p0 = lane - b.lo, q0 = -lane - b.lo;
+  if ((tpr & 3) == 0) {
+    // a thread's inputs are tpr (a multiple of 4) apart, so all lie in one phase
+    const int pp = p0 & 3, qp = q0 & 3;
+    const unsigned pa = b.grid + ((pp * b.ps) << 4) - (pp << 2), qa = b.grid + ((qp * b.ps) << 4) - (qp << 2) + 8;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int i = (p0 + r * tpr) & mask, k = (q0 - r * tpr) & mask;
+      float2 u = make_float2(0.f, 0.f), w = u;
+      if (i < b.n) u = lds2(pa + (i << 2));
+      if (k < b.n) w = lds2(qa + (k << 2));
+      v[r] = cadd(u, w);
+    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int i = (p0 + r * tpr) & mask, k = (q0 - r * tpr) & mask;
+      float2 u = make_float2(0.f, 0.f), w = u;
+      if (i < b.n) u = lds2(b.grid + (((i & 3) * b.ps + (i >> 2)) << 4));
+      if (k < b.n) w = lds2(b.grid + (((k & 3) * b.ps + (k >> 2)) << 4) + 8);
+      v[r] = cadd(u, w);
+    }
+  }
+  __syncthreads();
+  dft_reg<R, true>(v);
+  float2* dst = X + PADI(lane * R);
+#pragma unroll
+  for (int r = 0; r < R; ++r) dst[r] = v[r];
+  __syncthreads();
+}
+
+// Last pass of an adjoint row's inverse transform (radix R < 16, Ns = M/R,
+// 16/R butterflies j = lane + i M/16 per thread, outputs at m = j + r M/R)
+// with the crop fused: the outputs that hold samples n = (m + nt/2) mod M <
+// nt, times s_n = scale * prescale[n], go straight to dst[n].  At
+// oversampling 2 only half of each butterfly's outputs are kept (and
+// computed): r < R/4 and r >= 3R/4, for R = 2 the first output of j < M/4 and
+// the second of the others.
+template <int R>
+__device__ __forceinline__ void fft_last_crop(const float2* X, int M, int nt, int lane, int tpr,
+                                              const float2* __restrict__ tw, int twstride, float2* dst,
+                                              const float* __restrict__ prescale, float scale) {
+  constexpr int NB = kElemsPerThread / R;
+  const int MR = M / R, q4 = M >> 2, mask = M - 1, h = nt >> 1;
+  float2 v[NB][R];
+#pragma unroll
+  for (int i = 0; i < NB; ++i)
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[i][r] = X[PADI(lane + i * tpr + r * MR)];
+  TwBase<R> t0, t;
+  tw_load<R>(t0, tw, lane * twstride);
+  const bool two = M == 2 * nt;
+#pragma unroll
+  for (int i = 0; i < NB; ++i) {
+    const int j = lane + i * tpr;
+    if (i == 0) t = t0;
+    else tw_shift<R>(t, t0, i);
+    tw_apply<R, true>(v[i], t);
+    dft_reg<R, true>(v[i]);
+    if (two) {
+      if (R == 2) {
+        // j < M/4 for the first half of the butterflies (i < NB/2)
+        const int n = i < NB / 2 ? j + q4 : j + MR - 3 * q4;
+        const float2 y = i < NB / 2 ? v[i][0] : v[i][R - 1];
+        const float s = scale * __ldg(&prescale[n]);
+        dst[n] = make_float2(s * y.x, s * y.y);
+      } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          if (r >= R / 4 && r < 3 * R / 4) continue;
+          const int n = j + r * MR + (r < R / 4 ? q4 : -3 * q4);
+          const float s = scale * __ldg(&prescale[n]);
+          dst[n] = make_float2(s * v[i][r].x, s * v[i][r].y);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int n = (j + r * MR + h) & mask;
+        if (n < nt) {
+          const float s = scale * __ldg(&prescale[n]);
+          dst[n] = make_float2(s * v[i][r].x, s * v[i][r].y);
+        }
+      }
+    }
+  }
+}
+
+// Inverse length-M transform of an adjoint row with the crop fused: radix-16
+// passes, then the remaining radix (M/16 strided reads and unit-stride global
+// writes; as the first pass its scattered shared-memory writes conflicted
+// four to eight ways).  The last pass writes the outputs that hold samples
+// straight to dst (fft_last_crop).  When M is a power of 16 the last pass is
+// radix 16 (butterfly j = lane, outputs at m = j + r M/16); at oversampling 2
 // (M = 2 nt) only r = 0..3 (n = m + M/4) and r = 12..15 (n = m - 3M/4) are
 // kept, and only those 8 outputs are computed: with w = e^{+2 pi i/16},
 // A = inverse DFT8 of the even inputs and B of the odd,
 // Y[t] = A[t] + w^t B[t] (t = 0..3) and Y[t+8] = A[t] - w^t B[t] (t = 4..7).
+// BAND: the first pass reads the band grid.
+template <bool BAND>
 __device__ __forceinline__ void fft_inverse_crop(float2* X, int M, int mshift, int nt, int lane, int tpr,
                                                  const float2* __restrict__ tw, int twstride, float2* dst,
-                                                 const float* __restrict__ prescale, float scale, bool valid) {
-  int Ns = 1;
+                                                 const float* __restrict__ prescale, float scale, bool valid,
+                                                 const Band& band) {
+  if (BAND) fft_first_pass_band(X, M, lane, tpr, band);
+  else fft_pass<16, true, kLayoutPadded>(X, M, 1, lane, tpr, tw, twstride);
+  int Ns = 16;
   const int r0 = mshift & 3;
-  if (r0 == 3) {
-    fft_pass<8, true, kLayoutPadded>(X, M, 1, lane, tpr, tw, twstride);
-    Ns = 8;
-  } else if (r0 == 2) {
-    fft_pass<4, true, kLayoutPadded>(X, M, 1, lane, tpr, tw, twstride);
-    Ns = 4;
-  } else if (r0 == 1) {
-    fft_pass<2, true, kLayoutPadded>(X, M, 1, lane, tpr, tw, twstride);
-    Ns = 2;
-  }
   while (Ns * 16 < M) {
     fft_pass<16, true, kLayoutPadded>(X, M, Ns, lane, tpr, tw, twstride);
     Ns <<= 4;
   }
   if (!valid) return;
+  if (r0 != 0) {
+    if (r0 == 3) fft_last_crop<8>(X, M, nt, lane, tpr, tw, twstride, dst, prescale, scale);
+    else if (r0 == 2) fft_last_crop<4>(X, M, nt, lane, tpr, tw, twstride, dst, prescale, scale);
+    else fft_last_crop<2>(X, M, nt, lane, tpr, tw, twstride, dst, prescale, scale);
+    return;
+  }
   const int j = lane;
   float2 v[16];
   if ((Ns & 31) == 0) {
@@ -993,207 +1135,394 @@ __device__ __forceinline__ int floor_div(int a, int b) {  // b > 0
   return (a >= 0) ? a / b : -((-a + b - 1) / b);
 }
 
-// Adjoint of one row by node pairs spread by one warp (spread mode 3,
-// windowed methods, row slots of one or two warps).
-//
-// Phase 1: pair i holds the node pair +-x of one depth index (l = i + 1, or
-// j = i in forward-model mode), sorted by x: A[i] = (j0, fr, Q+) for the +x
-// node (x = j0 + fr) and B[i] = Q- for the -x node, each Q the node's input
-// value times the weight and the transpose of its phase, e^{+i pi nu} for +x
-// and its conjugate for -x.  The -x node is taken as (-j0 - 1) + (1 - fr), as
-// the forward gather takes it, so its tap q weighs w_{2H-1-q}(z), z = fr - 1/2:
-// one evaluation of the tap-pair polynomials serves both nodes.
-//
-// Phase 2: the row slot's first warp spreads all pairs into the grid X, 32
-// consecutive pairs at a time, one per lane (with a second warp in the slot,
-// as for M = 1024, that warp waits: a private grid for it cost more in
-// occupancy than it saved); pairs with equal j0 form a run (the list is
-// sorted), and for each tap pair and each of the four contributions (taps p
-// and 2H-1-p of +x and of -x) the run's terms are summed across its lanes
-// (segmented shuffle sum, only when the 32 pairs hold a run) and the run's
-// first lane adds the sum to its cell with a plain read-modify-write.  Within
-// one such step distinct runs have distinct j0, hence distinct cells (the 32
-// pairs span fewer than M - 2H cells, checked by the plan); a __syncwarp
-// separates the steps.  Every cell therefore receives its terms in a fixed
-// order: the result is bit-repeatable.
-// Returns whether the row is a mirror row (non-ZF input, both destinations).
-// ATOM (spread mode 4, rows of any number of warps): every warp of the slot
-// spreads its share of the 32-pair chunks, each run's sum added with
-// shared-memory atomics (the order of the additions into a cell varies).
-template <int H, bool ZF, bool ATOM = false>
-__device__ __forceinline__ bool adjoint_pairs(const RowProblem& P, const WindowPoly& W, int row, bool valid, int lane,
-                                              float2* X, float4* A) {
-  const int tpr = P.tpr, M = P.M, nt = P.nt, mask = M - 1;
+// Where a row's node pairs come from.
+struct PairSrc {
+  const float2* a;  // ZF: the row's depth spectrum; else the +k line of the half spectrum
+  const float2* b;  // else: the -k line
+  float2 S;         // |K_lat / 2 pi|^2 as float-float
+  bool mirror;      // the row has -nu nodes below the Nyquist entry
+};
+
+// Node pair i of a row: the nodes +-x of one depth index l = i + 1,
+// x = j0 + fr, and their values Q+ = qp, Q- = qn: the
+// input times the weight and the transpose of the node's phase, e^{+i pi nu}
+// for +x and its conjugate for -x.
+template <bool ZF>
+__device__ __forceinline__ void pair_node(const RowProblem& P, const PairSrc& src, int i, int& j0, float& fr,
+                                          float2& qp, float2& qn) {
   const int nzh = P.nz >> 1;
-  float2* B = reinterpret_cast<float2*>(A + nzh + 1);
-  bool mirror = true;
+  const int lp = i + 1;
+  const float4 zt = __ldg(&P.zt[lp]);
+  float rx;
+  node_position(src.S, zt, P.B2hi, P.B2lo, j0, fr, rx);
+  const float2 ph = node_phase(j0, fr, P.nt, P.M, P.nt_over_M);
+  float2 yp, yn;  // inputs of the two nodes, real weights applied
+  const float wt = P.wscale * zt.z * rx;
+  if (lp == nzh) {
+    // Nyquist: both nodes carry half the l = -nz/2 input
+    float2 y = src.a[lp];
+    if (!ZF && src.mirror) {
+      const float2 y2 = src.b[lp];
+      y = make_float2(y.x + y2.x, y.y - y2.y);
+    }
+    yp = yn = make_float2(0.5f * wt * y.x, 0.5f * wt * y.y);
+  } else if (ZF) {
+    const float2 y = src.a[lp], y2 = src.a[P.nz - lp];
+    yp = make_float2(wt * y.x, wt * y.y);
+    yn = make_float2(wt * y2.x, wt * y2.y);
+  } else {
+    const float2 y = src.a[lp];
+    yp = make_float2(2.0f * wt * y.x, 2.0f * wt * y.y);
+    yn = make_float2(0.f, 0.f);  // self-conjugate row: no -nu node below the Nyquist entry
+    if (src.mirror) {
+      const float2 y2 = src.b[lp];
+      yn = make_float2(2.0f * wt * y2.x, -2.0f * wt * y2.y);
+    }
+  }
+  qp = cmul(yp, ph);
+  qn = cmul(yn, make_float2(ph.x, -ph.y));
+}
+
+// Cells of a band grid: WIDE 16 bytes (two complex values that take the same
+// weights), else 8 bytes (one).
+template <bool WIDE>
+struct Cell {
+  float4 v;
+};
+template <>
+struct Cell<false> {
+  float2 v;
+};
+template <bool WIDE>
+constexpr int kCellShift = WIDE ? 4 : 3;
+
+template <bool WIDE>
+__device__ __forceinline__ Cell<WIDE> cell_zero() {
+  if constexpr (WIDE) return {make_float4(0.f, 0.f, 0.f, 0.f)};
+  else return {make_float2(0.f, 0.f)};
+}
+template <bool WIDE>
+__device__ __forceinline__ Cell<WIDE> cell_load(unsigned a) {
+  if constexpr (WIDE) return {lds4(a)};
+  else return {lds2(a)};
+}
+template <bool WIDE>
+__device__ __forceinline__ void cell_store(unsigned a, const Cell<WIDE>& c) {
+  if constexpr (WIDE) sts4(a, c.v);
+  else sts2(a, c.v);
+}
+template <bool WIDE>
+__device__ __forceinline__ Cell<WIDE> cell_add(const Cell<WIDE>& a, const Cell<WIDE>& b) {
+  if constexpr (WIDE) {
+    const float2 p = cadd(make_float2(a.v.x, a.v.y), make_float2(b.v.x, b.v.y));
+    const float2 n = cadd(make_float2(a.v.z, a.v.w), make_float2(b.v.z, b.v.w));
+    return {make_float4(p.x, p.y, n.x, n.y)};
+  } else {
+    return {cadd(a.v, b.v)};
+  }
+}
+// w q + g
+template <bool WIDE>
+__device__ __forceinline__ Cell<WIDE> cell_axpy(float w, const Cell<WIDE>& q, const Cell<WIDE>& g) {
+  const float2 ww = make_float2(w, w);
+  if constexpr (WIDE) {
+    const float2 p = fma2(ww, make_float2(q.v.x, q.v.y), make_float2(g.v.x, g.v.y));
+    const float2 n = fma2(ww, make_float2(q.v.z, q.v.w), make_float2(g.v.z, g.v.w));
+    return {make_float4(p.x, p.y, n.x, n.y)};
+  } else {
+    return {fma2(ww, q.v, g.v)};
+  }
+}
+template <bool WIDE>
+__device__ __forceinline__ Cell<WIDE> cell_shfl_down(const Cell<WIDE>& c, int d) {
+  const unsigned full = 0xffffffffu;
+  if constexpr (WIDE)
+    return {make_float4(__shfl_down_sync(full, c.v.x, d), __shfl_down_sync(full, c.v.y, d),
+                        __shfl_down_sync(full, c.v.z, d), __shfl_down_sync(full, c.v.w, d))};
+  else
+    return {make_float2(__shfl_down_sync(full, c.v.x, d), __shfl_down_sync(full, c.v.y, d))};
+}
+// Address of cell i (four phases, see Band).
+template <bool WIDE>
+__device__ __forceinline__ unsigned cell_at(const Band& b, int i) {
+  return b.grid + (((i & 3) * b.ps + (i >> 2)) << kCellShift<WIDE>);
+}
+
+// Tap addresses of one lane: tap t of a node whose first cell is cell0 sits at
+// a[t & 3] plus t / 4 cells (the four phases make every tap offset but four a
+// constant), or, for the first nspill taps, in the warp's spill.
+template <bool WIDE>
+struct BandTaps {
+  unsigned a[4];
+  unsigned spill;
+  int nspill;
+  __device__ __forceinline__ BandTaps(const Band& b, int cell0, unsigned spill_at, int ns)
+      : spill(spill_at), nspill(ns) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) a[j] = cell_at<WIDE>(b, cell0 + j);
+  }
+  __device__ __forceinline__ unsigned direct(int t) const { return a[t & 3] + ((t >> 2) << kCellShift<WIDE>); }
+  __device__ __forceinline__ unsigned at(int t) const {
+    return t < nspill ? spill + (t << kCellShift<WIDE>) : direct(t);
+  }
+};
+
+// Runs of lanes with equal j0 within a group of gw lanes (nodes are sorted).
+struct Runs {
+  bool head;    // first lane of its run
+  int first;    // that lane
+  int last;     // last lane of this lane's run
+  int maxrun;   // longest run of the warp
+  int mingap;   // least distance of neighbouring runs
+  bool sorted;  // rounding did not swap neighbouring nodes
+};
+__device__ __forceinline__ Runs find_runs(int j0, bool act, int gw) {
+  const unsigned full = 0xffffffffu;
+  const int l32 = threadIdx.x & 31;
+  const bool first = (l32 & (gw - 1)) == 0;
+  const int prev = __shfl_up_sync(full, j0, 1);
+  Runs r;
+  r.head = act && (first || prev != j0);
+  const unsigned heads = __ballot_sync(full, r.head), actm = __ballot_sync(full, act);
+  const unsigned stop = (heads | ~actm) & (0xfffffffeu << l32);  // the run ends before the next head or idle lane
+  r.last = stop ? __ffs(stop) - 2 : 31;
+  const unsigned mine = heads & (0xffffffffu >> (31 - l32));
+  r.first = mine ? 31 - __clz(mine) : l32;
+  r.maxrun = __reduce_max_sync(full, (unsigned)(r.head ? r.last - l32 + 1 : 0));
+  r.mingap = __reduce_min_sync(full, (unsigned)(r.head && !first ? max(j0 - prev, 0) : 1 << 20));
+  r.sorted = __all_sync(full, !(act && !first && prev > j0));
+  return r;
+}
+
+template <int H>
+__device__ __forceinline__ void tap_pair(const WindowPoly& W, int p, float z, float z2, float& wl, float& wh) {
+  float E = W.ce[p][kHalfCoef - 1], O = W.co[p][kHalfCoef - 1];
+#pragma unroll
+  for (int e = kHalfCoef - 2; e >= 0; --e) {
+    E = fmaf(E, z2, W.ce[p][e]);
+    O = fmaf(O, z2, W.co[p][e]);
+  }
+  wl = fmaf(z, O, E);
+  wh = fmaf(-z, O, E);
+}
+
+// Spreads one node per lane: q times its 2H weights.  Nodes on one cell (a run
+// of lanes) take turns; in each turn lanes write distinct cells at one tap,
+// neighbouring taps of different lanes may meet, so a __syncwarp separates
+// them.  Where all neighbouring nodes are two or more cells apart, two adjacent
+// taps of all lanes are still distinct cells and go together.  Long runs (nodes
+// crowd where the lateral frequency dominates) sum by shuffles instead: their
+// first lane adds.  The order of a cell's terms is fixed in every case.
+template <int H, bool WIDE>
+__device__ __forceinline__ void band_spread(const WindowPoly& W, const BandTaps<WIDE>& tp, int j0, float fr,
+                                            const Cell<WIDE>& q, bool act, int gw) {
+  const float z = fr - 0.5f, z2 = z * z;
+  const Runs r = find_runs(j0, act, gw);
+  float w[2 * H];
+#pragma unroll
+  for (int p = 0; p < H; ++p) tap_pair<H>(W, p, z, z2, w[p], w[2 * H - 1 - p]);
+  const bool ordered = r.sorted && r.maxrun <= 1;
+  if (ordered && r.mingap >= 2 && __all_sync(0xffffffffu, tp.nspill <= 0 || !act)) {
+#pragma unroll
+    for (int t = 0; t < 2 * H; t += 2) {
+      if (act) {
+        const Cell<WIDE> g0 = cell_load<WIDE>(tp.direct(t)), g1 = cell_load<WIDE>(tp.direct(t + 1));
+        cell_store<WIDE>(tp.direct(t), cell_axpy<WIDE>(w[t], q, g0));
+        cell_store<WIDE>(tp.direct(t + 1), cell_axpy<WIDE>(w[t + 1], q, g1));
+      }
+      __syncwarp();
+    }
+  } else if (r.sorted && r.maxrun > 4) {
+    const int l32 = threadIdx.x & 31;
+#pragma unroll
+    for (int t = 0; t < 2 * H; ++t) {
+      Cell<WIDE> v = cell_axpy<WIDE>(w[t], q, cell_zero<WIDE>());
+      for (int d = 1; d < r.maxrun; d <<= 1) {
+        const Cell<WIDE> u = cell_shfl_down<WIDE>(v, d);
+        if (l32 + d <= r.last) v = cell_add<WIDE>(v, u);
+      }
+      if (r.head) {
+        const unsigned a = tp.at(t);
+        cell_store<WIDE>(a, cell_add<WIDE>(cell_load<WIDE>(a), v));
+      }
+      __syncwarp();
+    }
+  } else {
+    // this lane's turn: its place in its run (any lane of its own where rounding swapped two neighbours)
+    const int turn = r.sorted ? (threadIdx.x & 31) - r.first : (threadIdx.x & (gw - 1));
+    const int turns = r.sorted ? r.maxrun : gw;
+    for (int k = 0; k < turns; ++k) {
+      const bool on = act && turn == k;
+#pragma unroll
+      for (int t = 0; t < 2 * H; ++t) {
+        if (on) {
+          const unsigned a = tp.at(t);
+          cell_store<WIDE>(a, cell_axpy<WIDE>(w[t], q, cell_load<WIDE>(a)));
+        }
+        __syncwarp();
+      }
+    }
+  }
+}
+
+// A row's (or unit's) sorted nodes divided over its warps, and the part of the
+// band each warp adds to.  Cells at or below the predecessor's last cell go to
+// the warp's own spill of kSpill cells and are merged after a barrier; all
+// others the warp owns alone, so it zeroes them and begins without a barrier.
+template <int H>
+struct BandPart {
+  static constexpr int kSpill = 2 * H + 4;
+  int nw, wa, w;       // warps, warps with nodes, this warp
+  int gw, l;           // lanes per row in a warp, this lane's place
+  int n0, n1;          // this warp's nodes
+  int lo_w, hi_prev;   // first cell of this warp's nodes, last cell of its predecessor's
+  unsigned spills, spill_w;
+  int2* bnd;           // first cell and last cell per warp (shared memory)
+};
+
+// Sets up the parts and zeroes the cells this warp owns and its spill.
+// position(i): cell index j0 of node i.  One cell to spare on either side,
+// should rounding swap two neighbouring nodes.
+template <int H, bool WIDE, typename Pos>
+__device__ __forceinline__ void band_begin(BandPart<H>& b, Band& band, char* slot, int ps, int np, int lane, int threads,
+                                           Pos position) {
+  constexpr int kSpill = BandPart<H>::kSpill, kShift = kCellShift<WIDE>;
+  b.nw = threads > 32 ? threads >> 5 : 1;
+  b.gw = threads < 32 ? threads : 32;
+  b.w = threads > 32 ? lane >> 5 : 0;
+  b.l = lane & (b.gw - 1);
+  b.wa = min(b.nw, (np + 31) >> 5);  // warps with a full chunk of nodes each
+  const bool on = b.w < b.wa;
+  b.n0 = on ? np * b.w / b.wa : np;
+  b.n1 = on ? np * (b.w + 1) / b.wa : np;
+  band.grid = smem_addr(slot);
+  band.ps = ps;
+  band.lo = 0;
+  band.n = 0;
+  b.spills = band.grid + ((4 * ps) << kShift);
+  b.spill_w = b.spills + ((b.w * kSpill) << kShift);
+  b.bnd = reinterpret_cast<int2*>(slot + ((4 * ps + (b.nw > 1 ? b.nw * kSpill : 0)) << kShift));
+  // lanes 0 .. 3: first node of the row, last of this warp, first of this warp, last of the predecessor
+  int j = 0;
+  if (on && b.l < 4) j = position(b.l == 0 ? 0 : b.l == 1 ? b.n1 - 1 : b.l == 2 ? b.n0 : max(b.n0 - 1, 0));
+  const unsigned full = 0xffffffffu;
+  const int j_row = __shfl_sync(full, j, 0, b.gw), j_last = __shfl_sync(full, j, 1, b.gw);
+  const int j_first = b.nw > 1 ? __shfl_sync(full, j, 2) : j_row, j_prev = b.nw > 1 ? __shfl_sync(full, j, 3) : j_row;
+  band.lo = j_row - H;
+  b.lo_w = j_first - H;
+  b.hi_prev = b.w > 0 ? j_prev + H + 1 : -(1 << 30);
+  if (on) {
+    const int hi = j_last + H + 1;
+    if (b.l == 0) b.bnd[b.w] = make_int2(b.lo_w, hi);
+    const Cell<WIDE> zero = cell_zero<WIDE>();
+    for (int c = (b.w > 0 ? b.hi_prev + 1 - band.lo : 0) + b.l; c <= hi - band.lo; c += b.gw)
+      cell_store<WIDE>(cell_at<WIDE>(band, c), zero);
+    if (b.nw > 1 && b.l < kSpill) cell_store<WIDE>(b.spill_w + (b.l << kShift), zero);
+  }
+  __syncwarp();
+}
+
+// After the spread's barrier: merges the spills (a cell spilled by several
+// warps is summed by the first of them, in warp order) and sets band.n.
+// fold: cells `fold` apart are one grid value (bands longer than that, for
+// coarse time steps or tiny grids, are folded).  uniform over the CTA: nw, ps.
+template <int H, bool WIDE>
+__device__ __forceinline__ void band_end(const BandPart<H>& b, Band& band, int lane, int threads, int fold) {
+  constexpr int kSpill = BandPart<H>::kSpill, kShift = kCellShift<WIDE>;
+  if (b.wa > 0) {
+    band.lo = b.bnd[0].x;  // (warps without nodes do not have it)
+    band.n = b.bnd[b.wa - 1].y + 1 - band.lo;
+  }
+  if (b.nw > 1) {
+    const int c = b.lo_w + b.l;
+    if (b.w > 0 && b.w < b.wa && b.l < kSpill && c <= b.hi_prev && (b.w == 1 || c > b.bnd[b.w - 2].y)) {
+      const unsigned a = cell_at<WIDE>(band, c - band.lo);
+      Cell<WIDE> s = cell_load<WIDE>(a);
+      for (int v = b.w; v < b.wa && c >= b.bnd[v].x; ++v)
+        s = cell_add<WIDE>(s, cell_load<WIDE>(b.spills + ((v * kSpill + c - b.bnd[v].x) << kShift)));
+      cell_store<WIDE>(a, s);
+    }
+    __syncthreads();
+  }
+  if (4 * band.ps > fold) {
+    for (int i = lane; i < fold && i < band.n - fold; i += threads) {
+      const unsigned a = cell_at<WIDE>(band, i);
+      Cell<WIDE> g = cell_load<WIDE>(a);
+      for (int k = i + fold; k < band.n; k += fold) g = cell_add<WIDE>(g, cell_load<WIDE>(cell_at<WIDE>(band, k)));
+      cell_store<WIDE>(a, g);
+    }
+    __syncthreads();
+    band.n = min(band.n, fold);
+  }
+}
+
+// Adjoint of one row by node pairs (spread mode 3, windowed methods): the
+// transpose of the gather, deterministic and without atomics.
+//
+// The -x node of a pair is taken as (-j0 - 1) + (1 - fr), as the forward
+// gather takes it, so its tap at cell -c weighs what the +x node's tap at cell
+// c weighs.  Both therefore add with one weight to one 16-byte (WIDE) cell of the
+// band grid (struct Band), which covers only the cells the row's nodes reach:
+// one read and one write of 16 bytes per tap and pair, half the accesses of
+// two separate complex cells.  The first inverse FFT pass reads the grid
+// values from the band.
+//
+// The row's warps take contiguous blocks of the sorted pairs (BandPart).  A
+// pair's values are formed right before they are spread (no list in shared
+// memory).
+//
+// What bounds it: shared-memory accesses, 32 bytes per tap and pair.  The
+// lists and float atomics it replaces held one CTA per SM for long rows and
+// serialised on equal cells.
+template <int H, bool ZF>
+__device__ __forceinline__ bool adjoint_band(const RowProblem& P, const WindowPoly& W, int row, bool valid, int lane,
+                                             float2* X, Band& band) {
+  PairSrc src{nullptr, nullptr, make_float2(0.f, 0.f), true};
   int np = 0;
   if (valid) {
-    const float2* Zs = P.fh + (size_t)row * P.zstride;  // ZF: the row's depth spectrum Fbar[l mod nz]
-    if (ZF && P.qmode) {
-      // forward model: pair j (j = 0..nz/2) carries c_j / 2 on both nodes,
-      // c_j = F[j] + F[-j] (F[0], F[nz/2] alone), stored by the depth stage at
-      // Zs[j]; wscale holds 1 / (2 n_lat nz)
-      const float2 S = P.rowS[row];
-      np = nzh + 1;
-      for (int j = lane; j <= nzh; j += tpr) {
-        const float4 zt = __ldg(&P.zt[j]);
-        int j0;
-        float fr, rx;
-        node_position(S, zt, P.B2hi, P.B2lo, j0, fr, rx);
-        const float2 y = Zs[j];
-        const float2 pb = make_float2(P.wscale * y.x, P.wscale * y.y);
-        const float2 ph = node_phase(j0, fr, nt, M, P.nt_over_M);
-        const float2 qp = cmul(pb, ph), qn = cmul(pb, make_float2(ph.x, -ph.y));
-        A[j] = make_float4(__int_as_float(j0), fr, qp.x, qp.y);
-        B[j] = qn;
-      }
+    np = P.nz >> 1;
+    if (ZF) {
+      src.a = P.fh + (size_t)row * P.zstride;
+      src.S = P.rowS[row];
     } else {
-      RowGeom rg;
-      const float2* in1 = nullptr;
-      const float2* in2 = nullptr;
-      if (ZF) {
-        rg.S = P.rowS[row];
-      } else {
-        rg = row_geom(P, row);
-        mirror = rg.mirror;
-        in1 = P.fh + (size_t)rg.d1 * P.lz;
-        in2 = P.fh + (size_t)rg.d2 * P.lz;
-      }
-      np = nzh;
-      for (int i = lane; i < nzh; i += tpr) {
-        const int lp = i + 1;
-        const float4 zt = __ldg(&P.zt[lp]);
-        int j0;
-        float fr, rx;
-        node_position(rg.S, zt, P.B2hi, P.B2lo, j0, fr, rx);
-        const float wt = P.wscale * zt.z * rx;
-        const float2 ph = node_phase(j0, fr, nt, M, P.nt_over_M);
-        const float2 phc = make_float2(ph.x, -ph.y);
-        float2 qp, qn;
-        if (lp == nzh) {
-          // Nyquist: both nodes carry half the l = -nz/2 input
-          float2 y;
-          if (ZF) {
-            y = Zs[nzh];
-          } else {
-            y = in1[lp];
-            if (mirror) {
-              const float2 y2 = in2[lp];
-              y.x += y2.x;
-              y.y -= y2.y;
-            }
-          }
-          const float2 pb = make_float2(0.5f * wt * y.x, 0.5f * wt * y.y);
-          qp = cmul(pb, ph);
-          qn = cmul(pb, phc);
-        } else if (ZF) {
-          const float2 y = Zs[lp], y2 = Zs[P.nz - lp];
-          qp = cmul(make_float2(wt * y.x, wt * y.y), ph);
-          qn = cmul(make_float2(wt * y2.x, wt * y2.y), phc);
-        } else {
-          const float2 y = in1[lp];
-          qp = cmul(make_float2(2.0f * wt * y.x, 2.0f * wt * y.y), ph);
-          if (mirror) {
-            const float2 y2 = in2[lp];
-            qn = cmul(make_float2(2.0f * wt * y2.x, -2.0f * wt * y2.y), phc);
-          } else {
-            qn = make_float2(0.f, 0.f);  // self-conjugate row: no -nu node below the Nyquist entry
-          }
-        }
-        A[i] = make_float4(__int_as_float(j0), fr, qp.x, qp.y);
-        B[i] = qn;
-      }
+      const RowGeom rg = row_geom(P, row);
+      src.a = P.fh + (size_t)rg.d1 * P.lz;
+      src.b = P.fh + (size_t)rg.d2 * P.lz;
+      src.S = rg.S;
+      src.mirror = rg.mirror;
     }
   }
-  __syncthreads();  // pair lists complete (every row slot)
-  // the row slot's first warp spreads every pair; a second warp (rows of
-  // 64 threads) waits at the barrier below
-  const int w = lane >> 5, l32 = lane & 31;
-  float2* G = X;
-  if (ATOM) {
-    for (int g = lane; g < M; g += tpr) G[PADI(g)] = make_float2(0.f, 0.f);
-    __syncthreads();  // the grid is zero before any warp adds to it
-  } else if (w == 0) {
-    for (int g = l32; g < M; g += 32) G[PADI(g)] = make_float2(0.f, 0.f);
-    __syncwarp();
+  BandPart<H> part;
+  band_begin<H, true>(part, band, reinterpret_cast<char*>(X), P.band_ps, np, lane, P.tpr, [&](int i) {
+    int j0;
+    float fr, rx;
+    node_position(src.S, __ldg(&P.zt[i + 1]), P.B2hi, P.B2lo, j0, fr, rx);
+    return j0;
+  });
+  // chunks: uniform over the warp (rows sharing a warp have equal counts, or none)
+  const int cn = __reduce_max_sync(0xffffffffu, (unsigned)(part.n1 - part.n0));
+  for (int c0 = 0; c0 < cn; c0 += part.gw) {
+    const int i = part.n0 + c0 + part.l;
+    const bool act = i < part.n1;
+    int j0 = 0;
+    float fr = 0.5f;
+    float2 qp = make_float2(0.f, 0.f), qn = qp;
+    if (act) pair_node<ZF>(P, src, i, j0, fr, qp, qn);
+    const int c = j0 - H + 1;  // first cell
+    const BandTaps<true> tp(band, c - band.lo, part.spill_w + ((c - part.lo_w) << 4), part.hi_prev + 1 - c);
+    band_spread<H, true>(W, tp, j0, fr, Cell<true>{make_float4(qp.x, qp.y, qn.x, qn.y)}, act, part.gw);
   }
-  if (valid && (ATOM || w == 0)) {
-    const unsigned full = 0xffffffffu;
-    const int p1 = np;
-    const int c_first = ATOM ? 32 * w : 0, c_step = ATOM ? tpr : 32;
-    for (int c0 = c_first; c0 < p1; c0 += c_step) {
-      const int i = c0 + l32;
-      const bool act = i < p1;
-      const float4 a = act ? A[i] : make_float4(0.f, 0.5f, 0.f, 0.f);
-      const float2 b = act ? B[i] : make_float2(0.f, 0.f);
-      const int j0 = __float_as_int(a.x);
-      const int prev = __shfl_up_sync(full, j0, 1);
-      const bool head = act && (l32 == 0 || prev != j0);
-      const unsigned heads = __ballot_sync(full, head);
-      const unsigned actm = __ballot_sync(full, act);
-      // last lane of this lane's run
-      const unsigned later = heads & (0xfffffffeu << l32);
-      const int last = later ? __ffs(later) - 2 : 31 - __clz(actm);
-      const int span = head ? last - l32 + 1 : 0;
-      const int maxrun = __reduce_max_sync(full, (unsigned)span);
-      const float2 qp = make_float2(a.z, a.w);
-      const float z = a.y - 0.5f, z2 = z * z;
-      const int cp0 = j0 - H + 1;  // cell of tap 0 of +x
-      const int cn0 = -j0 - H;     // cell of tap 0 of -x
-#pragma unroll
-      for (int p = 0; p < H; ++p) {
-        float E = W.ce[p][kHalfCoef - 1], O = W.co[p][kHalfCoef - 1];
-#pragma unroll
-        for (int e = kHalfCoef - 2; e >= 0; --e) {
-          E = fmaf(E, z2, W.ce[p][e]);
-          O = fmaf(O, z2, W.co[p][e]);
-        }
-        const float wl = fmaf(z, O, E), wh = fmaf(-z, O, E);
-        // taps p and 2H-1-p of +x (weights wl, wh); of -x (wh, wl)
-        float2 c[4] = {mul2(make_float2(wl, wl), qp), mul2(make_float2(wh, wh), qp), mul2(make_float2(wh, wh), b),
-                       mul2(make_float2(wl, wl), b)};
-        if (maxrun > 1) {
-          for (int d = 1; d < maxrun; d <<= 1) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const float tx = __shfl_down_sync(full, c[k].x, d);
-              const float ty = __shfl_down_sync(full, c[k].y, d);
-              if (l32 + d <= last) {
-                c[k].x += tx;
-                c[k].y += ty;
-              }
-            }
-          }
-        }
-        const int cell[4] = {cp0 + p, cp0 + 2 * H - 1 - p, cn0 + p, cn0 + 2 * H - 1 - p};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          if (head) {
-            float2* q = G + PADI(cell[k] & mask);
-            if (ATOM) {
-              atomicAdd(&q->x, c[k].x);
-              atomicAdd(&q->y, c[k].y);
-            } else {
-              *q = cadd(*q, c[k]);
-            }
-          }
-          if (!ATOM) __syncwarp();
-        }
-      }
-    }
-  }
-  __syncthreads();  // the grid is complete
-  return mirror;
+  __syncthreads();  // every warp's cells and spills are complete
+  band_end<H, true>(part, band, lane, P.tpr, P.M);
+  return src.mirror;
 }
 
 // The adjoint row kernel with the pair spread (spread mode 3), a kernel of its
 // own so that its register allocation does not carry the other schemes.
-template <int H, bool ZF, bool ATOM>
+template <int H, bool ZF>
 __global__ void __launch_bounds__(1024) row_adjoint_pairs_kernel(RowLaunch L, WindowPoly W) {
   extern __shared__ float2 smem[];
   __shared__ int s_item;
-  float4* nodes_all = reinterpret_cast<float4*>(smem + L.fft_region);
   for (int item = blockIdx.x; item < L.nitems; item = next_item(L, &s_item)) {
     const WorkItem wi = L.items[item];
     const RowProblem& P = L.problems[wi.problem];
@@ -1202,12 +1531,139 @@ __global__ void __launch_bounds__(1024) row_adjoint_pairs_kernel(RowLaunch L, Wi
     const int lane = threadIdx.x - slot * tpr;
     const int row = wi.row0 + slot;
     const bool valid = row < P.rows;
-    float2* X = smem + slot * P.slot;
-    float4* N = nodes_all + slot * (P.nz + 2);
-    const bool mirror = adjoint_pairs<H, ZF, ATOM>(P, W, row, valid, lane, X, N);
+    float2* X = smem + slot * P.band_slot;
+    Band band;
+    const bool mirror = adjoint_band<H, ZF>(P, W, row, valid, lane, X, band);
     const float scale = (valid && !ZF && mirror) ? 0.5f : 1.0f;
     float2* dst = const_cast<float2*>(P.pt) + (size_t)(valid ? row : 0) * nt;
-    fft_inverse_crop(X, M, P.mshift, nt, lane, tpr, L.tw, L.Mmax >> P.mshift, dst, P.prescale, scale, valid);
+    fft_inverse_crop<true>(X, M, P.mshift, nt, lane, tpr, L.tw, L.Mmax >> P.mshift, dst, P.prescale, scale, valid,
+                           band);
+  }
+}
+
+// Forward-model row kernel (the operator Q of Sec. 2 on a padded periodic
+// box).  A row's samples are g_n = sum_j c_j cos(2 pi nu_j n / nt), j =
+// 0..nz/2, nu_j >= 0 the frequency of |K| (j = 0 included: its frequency is
+// the lateral |K|); Zs[j] holds c_j.
+//
+// The sum is even in n, so it is taken as a NUFFT over the interval (-nt, nt),
+// centred at n = 0: a grid of 2M cells at the half-integers m + 1/2, nodes at
+// x' = 2 x - 1/2, real window weights and no node phases; the mirrored nodes
+// are the reflection m -> -1 - m.  What is left is a cosine transform of M
+// cells (type II), taken as one complex transform of length M: with V1 the sum
+// over the nodes (no mirror), v[e] = V1[2e] + V1[-1-2e] (indices modulo 2M) and
+// its transform V,
+//   g_n = t_n V[n] + conj(t_n) V[M - n],   t_n = s_n e^{-i pi n / (2M)},
+// s_n the window's prescale over the doubled interval.  Against the node pairs
+// of the adjoint (two nodes with phases per index) this halves the values
+// spread and drops a sine and cosine per node.
+//
+// PAIR (3-D): rows k1 and -k1 have the same |K| and so the same nodes; a unit
+// of 2 tpr threads spreads both rows' values with one set of weights into
+// 16-byte cells, then transforms one row with each half of its threads.
+//
+// What bounds it: instruction issue (about a third of it node positions and
+// weights) and shared-memory accesses.
+template <int H, bool PAIR>
+__global__ void __launch_bounds__(1024) row_model_kernel(RowLaunch L, WindowPoly W) {
+  extern __shared__ float2 smem[];
+  __shared__ int s_item;
+  constexpr int kShift = kCellShift<PAIR>;
+  for (int item = blockIdx.x; item < L.nitems; item = next_item(L, &s_item)) {
+    const WorkItem wi = L.items[item];
+    const RowProblem& P = L.problems[wi.problem];
+    const int tpr = P.tpr, M = P.M, nzh = P.nz >> 1;
+    const int tpu = PAIR ? 2 * tpr : tpr;
+    const int slot = threadIdx.x / tpu;
+    const int lane_u = threadIdx.x - slot * tpu;
+    const int sub = PAIR ? lane_u / tpr : 0, lane = lane_u - sub * tpr;
+    const int unit = wi.row0 + slot;
+    const bool valid = unit < (PAIR ? (P.n1 / 2 + 1) * (P.n2 / 2 + 1) : P.rows);
+    int row_b = -1;  // the partner row (k1, k2) -> (-k1, k2)
+    if (PAIR && valid) {
+      const int half1 = P.n2 / 2 + 1, i1 = unit / half1;
+      if (i1 > 0 && i1 < P.n1 / 2) row_b = (P.n1 - i1) * half1 + (unit - i1 * half1);
+    }
+    float2* U = smem + (size_t)slot * P.model_slot;
+    const float2* za = P.fh + (size_t)(valid ? unit : 0) * P.zstride;
+    const float2* zb = P.fh + (size_t)(row_b >= 0 ? row_b : 0) * P.zstride;
+    const float2 S = valid ? P.rowS[unit] : make_float2(0.f, 0.f);
+    // cell index and fraction of node i on the half-integer grid
+    auto node = [&](int i, int& j0, float& fr) {
+      float rx;
+      node_position(S, __ldg(&P.zt[i]), 4.0f * P.B2hi, 4.0f * P.B2lo, j0, fr, rx);
+      fr -= 0.5f;
+      if (fr < 0.0f) {
+        fr += 1.0f;
+        j0 -= 1;
+      }
+    };
+    Band band;
+    BandPart<H> part;
+    band_begin<H, PAIR>(part, band, reinterpret_cast<char*>(U), P.model_ps, valid ? nzh + 1 : 0, lane_u, tpu, [&](int i) {
+      int j0;
+      float fr;
+      node(i, j0, fr);
+      return j0;
+    });
+    const int cn = __reduce_max_sync(0xffffffffu, (unsigned)(part.n1 - part.n0));
+    for (int c0 = 0; c0 < cn; c0 += part.gw) {
+      const int i = part.n0 + c0 + part.l;
+      const bool act = i < part.n1;
+      int j0 = 0;
+      float fr = 0.5f;
+      Cell<PAIR> q = cell_zero<PAIR>();
+      if (act) {
+        const float2 ya = __ldg(za + i);
+        if constexpr (PAIR) {
+          const float2 yb = row_b >= 0 ? __ldg(zb + i) : make_float2(0.f, 0.f);
+          q.v = make_float4(P.wscale * ya.x, P.wscale * ya.y, P.wscale * yb.x, P.wscale * yb.y);
+        } else {
+          q.v = make_float2(P.wscale * ya.x, P.wscale * ya.y);
+        }
+        node(i, j0, fr);
+      }
+      const int c = j0 - H + 1;
+      const BandTaps<PAIR> tp(band, c - band.lo, part.spill_w + ((c - part.lo_w) << kShift), part.hi_prev + 1 - c);
+      band_spread<H, PAIR>(W, tp, j0, fr, q, act, part.gw);
+    }
+    __syncthreads();
+    band_end<H, PAIR>(part, band, lane_u, tpu, 2 * M);
+    // first pass (radix 16): element e = lane + r M/16; a thread's cells lie 2 M/16 (a multiple of 4) apart, in one phase
+    float2* X = U + (PAIR ? sub * P.slot : 0);
+    {
+      constexpr int R = 16;
+      float2 v[R];
+      const int mask = 2 * M - 1;
+      const int p0 = 2 * lane - band.lo, q0 = -1 - 2 * lane - band.lo;
+      const int pp = p0 & 3, qp = q0 & 3;
+      const unsigned half = sub << 3;
+      const unsigned pa = band.grid + ((pp * band.ps) << kShift) + half;
+      const unsigned qa = band.grid + ((qp * band.ps) << kShift) + half;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int i = (p0 + 2 * r * tpr) & mask, k = (q0 - 2 * r * tpr) & mask;
+        float2 a = make_float2(0.f, 0.f), b = a;
+        if (i < band.n) a = lds2(pa + ((i >> 2) << kShift));
+        if (k < band.n) b = lds2(qa + ((k >> 2) << kShift));
+        v[r] = cadd(a, b);
+      }
+      __syncthreads();  // the band is read before its memory takes the transform
+      first_pass_regs<false>(X, v, lane);
+    }
+    __syncthreads();
+    fft_rest<false, kLayoutFlat>(X, M, P.mshift, lane, tpr, L.tw, L.Mmax >> P.mshift);
+    const int row = sub ? row_b : (valid ? unit : -1);
+    if (row >= 0) {
+      float2* dst = const_cast<float2*>(P.pt) + (size_t)row * P.nt;
+      for (int n = lane; n < P.nt; n += tpr) {
+        const float2 t = __ldg(&P.model_tab[n]);
+        const float2 a = X[n], b = X[(M - n) & (M - 1)];
+        // t a + conj(t) b
+        dst[n] = fma2(make_float2(t.x, t.x), cadd(a, b),
+                      mul2(make_float2(t.y, t.y), make_float2(b.y - a.y, a.x - b.x)));
+      }
+    }
   }
 }
 
@@ -1512,7 +1968,8 @@ __global__ void __launch_bounds__(1024) row_adjoint_kernel(RowLaunch L, WindowPo
     __syncthreads();
     const float scale = (valid && !ZF && rg.mirror) ? 0.5f : 1.0f;
     float2* dst = const_cast<float2*>(P.pt) + (size_t)(valid ? row : 0) * nt;
-    fft_inverse_crop(X, M, P.mshift, nt, lane, tpr, L.tw, L.Mmax >> P.mshift, dst, P.prescale, scale, valid);
+    fft_inverse_crop<false>(X, M, P.mshift, nt, lane, tpr, L.tw, L.Mmax >> P.mshift, dst, P.prescale, scale, valid,
+                            Band{});
   }
 }
 
