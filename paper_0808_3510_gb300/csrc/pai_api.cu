@@ -958,7 +958,7 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     P->threads = T;
     size_t region = 0;
     for (int i = 0; i < count; ++i)
-      region = std::max(region, (size_t)rp[i].rpc * (size_t)rp[i].slot * sizeof(float2));
+      region = std::max(region, (size_t)rp[i].rpc * (size_t)rp[i].slot32 * sizeof(float2));
     P->fft_region = (int)(region / sizeof(float2));
     P->smem_fwd = region;
     if (P->smem_fwd > (size_t)smem_optin) return PAI_ERR_UNSUPPORTED;
@@ -984,7 +984,7 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     for (int i = 0; i < count; ++i) {
       const int rpc = T / P->probs[i].tpr;
       node_cap = std::max(node_cap, rpc * (P->probs[i].g.nz + 2));
-      region = std::max(region, (size_t)rpc * (size_t)rp[i].slot * sizeof(float2));
+      region = std::max(region, (size_t)rpc * (size_t)rp[i].slot32 * sizeof(float2));
     }
     P->threads_adj = T;
     P->fft_region_adj = (int)(region / sizeof(float2));

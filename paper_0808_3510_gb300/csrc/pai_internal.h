@@ -61,7 +61,8 @@ struct RowProblem {
   int n1, n2, rows;
   int tpr;                 // threads per row in the FFT = M / kElemsPerThread
   int rpc;                 // rows per CTA work item
-  int slot;                // complex values per row slot in shared memory (row_slot_stride(M))
+  int slot;                // complex values per row slot in shared memory (row_slot_stride(M)): band spreads
+  int slot32;           // the same with one pad per 32: forward kernel and the adjoint's list spreads
   float B2hi, B2lo;        // (M c dt)^2 as float-float: node x = B sqrt(S + az)
   float wscale;            // 2 c dt/dz * B / (n1 n2 nz): W = wscale * kz / x
   float nt_over_M;         // for the node phase
@@ -73,6 +74,7 @@ struct RowProblem {
                            // the rows hold c_j, j = 0..nz/2, nz/2 + 2 values apart)
   int band_ps, band_slot;  // adjoint pair spread: cells per phase of the band grid, complex values per row slot
   int model_ps, model_slot;  // the same for the forward-model row kernel (per unit of one or two rows)
+  int model_dense;           // neighbouring nodes are at most two cells apart there
   const float2* model_tab;   // forward-model row kernel: [nt] prescale times e^{-i pi n / (2M)}
   int paired;              // 2-D, forward: pt holds Z[k][m] (k < nx = n2, m < nt/2, row stride nt/2), the
                            // lateral DFT of the sample pairs p[x][2m] + i p[x][2m+1]; the forward row kernel
@@ -105,9 +107,11 @@ struct RowLaunch {
   int paired;                  // forward: some problem is in the paired layout (RowProblem::paired)
 };
 
-// Complex values one row slot needs: the padded FFT layout (one pad per 32)
-// and the flat layout with 2*kMaxH ghost cells must both fit.
-__host__ __device__ inline int row_slot_stride(int M) { return M + ((M >> 5) > 2 * kMaxH ? (M >> 5) : 2 * kMaxH); }
+// Complex values one row slot needs: the padded FFT layout (one pad per 16 at
+// most) and the flat layout with 2*kMaxH ghost cells must both fit.
+__host__ __device__ inline int row_slot_stride(int M, int pad = 4) {
+  return M + ((M >> pad) > 2 * kMaxH ? (M >> pad) : 2 * kMaxH);
+}
 
 // Host-side window math (FP64), pai_window.cpp
 double bessel_i0(double x);

@@ -20,9 +20,18 @@
 
 namespace pai {
 
-// Complex values per FFT slot: padded layout plus a shift of 4 values so the
-// FP slots start in different shared-memory banks.
-__host__ __device__ inline int lateral_slot(int L) { return L + (L >> 5) + 4; }
+// Complex values per FFT slot of FP column slots side by side: the padded
+// layout, with the slots 16 / FP (mod 16) values apart: the 16 lanes of a
+// half-warp in the load and store phases, FP columns times 16 / FP consecutive
+// elements, then fall on 16 different banks, in the first pass's writes too
+// (17 x0 + r).  (One pad per 32 and a shift of 4 made those accesses two- to
+// four-way conflicts.)
+__host__ __device__ constexpr int lateral_slot(int L, int FP) {
+  const int s = L + (L >> 4);
+  return s + (16 / FP - s % 16 + 16) % 16;
+}
+// The same for lines handled one after another (rows_fft_kernel, rows_fold_kernel).
+__host__ __device__ constexpr int rows_slot(int L) { return L + (L >> 4); }
 
 enum : int { kLatR2C = 0, kLatC2R = 1, kLatC2C = 2, kLatC2CInv = 3 };
 
@@ -49,7 +58,7 @@ __global__ void __launch_bounds__(1024) lateral_kernel(const void* vin, void* vo
   extern __shared__ float2 smem[];
   constexpr bool kInv = (KIND == kLatC2R || KIND == kLatC2CInv);
   const int tpr = L / kElemsPerThread;
-  const int S = lateral_slot(L);
+  const int S = lateral_slot(L, FP);
   const int T = blockDim.x;
   const int f = threadIdx.x % FP;  // column group of this thread in the load / store phases
   const int x0 = threadIdx.x / FP;
@@ -100,11 +109,11 @@ __global__ void __launch_bounds__(1024) lateral_kernel(const void* vin, void* vo
       const float4 ab = abv[i];
       if (k == 0 || k == half) {
         // self-conjugate bins: only the real parts enter a C2R
-        Z[PADI(k)] = make_float2(ab.x, ab.z);
+        Z[padi(k)] = make_float2(ab.x, ab.z);
       } else {
         // Z[k] = A[k] + i B[k];  Z[L-k] = conj A[k] + i conj B[k]
-        Z[PADI(k)] = make_float2(ab.x - ab.w, ab.y + ab.z);
-        Z[PADI(L - k)] = make_float2(ab.x + ab.w, ab.z - ab.y);
+        Z[padi(k)] = make_float2(ab.x - ab.w, ab.y + ab.z);
+        Z[padi(L - k)] = make_float2(ab.x + ab.w, ab.z - ab.y);
       }
     }
   }
@@ -166,7 +175,7 @@ int lateral_slots_per_cta(int L) {
   return fp;
 }
 
-size_t lateral_smem_bytes(int L) { return (size_t)lateral_slots_per_cta(L) * lateral_slot(L) * sizeof(float2); }
+size_t lateral_smem_bytes(int L) { return (size_t)lateral_slots_per_cta(L) * lateral_slot(L, lateral_slots_per_cta(L)) * sizeof(float2); }
 
 bool lateral_supported(int L, int C) {
   if (L < 32 || (L & (L - 1)) != 0) return false;
@@ -248,7 +257,7 @@ __global__ void __launch_bounds__(1024) rows_fft_kernel(float2* data, int L, int
   const int rpc = blockDim.x / tpr;
   const int row = blockIdx.x * rpc + slot;
   const bool valid = row < rows;
-  float2* X = smem + slot * lateral_slot(L);
+  float2* X = smem + slot * rows_slot(L);
   float2* line = data + (size_t)(valid ? row : 0) * L;
   {
     constexpr int R = 16;
@@ -260,7 +269,7 @@ __global__ void __launch_bounds__(1024) rows_fft_kernel(float2* data, int L, int
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int idx = lane * R + r;
-      X[PADI(idx)] = v[r];
+      X[padi(idx)] = v[r];
     }
   }
   __syncthreads();
@@ -277,7 +286,7 @@ cudaError_t launch_rows_c2c(float2* data, int L, int rows, bool inverse, const f
   const int tpr = L / kElemsPerThread;
   const int threads = tpr > 128 ? tpr : 128;  // (128 measured 1.5 us faster than 256 per 256^3 depth stage)
   const int rpc = threads / tpr;
-  const size_t smem = (size_t)rpc * lateral_slot(L) * sizeof(float2);
+  const size_t smem = (size_t)rpc * rows_slot(L) * sizeof(float2);
   const int ctas = (rows + rpc - 1) / rpc;
   cudaError_t e;
   if (inverse) {
@@ -306,19 +315,37 @@ __global__ void __launch_bounds__(1024) rows_fold_kernel(const float2* __restric
   const int lane = threadIdx.x - slot * tpr;
   const int row = blockIdx.x * (blockDim.x / tpr) + slot;
   const bool valid = row < rows;
-  float2* X = smem + slot * lateral_slot(L);
-  {
-    const float2* line = in + (size_t)(valid ? row : 0) * n;
-    float2 v[kElemsPerThread];
+  float2* X = smem + slot * rows_slot(L);
+  const float2* line = in + (size_t)(valid ? row : 0) * n;
+  float2 v[kElemsPerThread];
+  if (2 * n <= L && mshift >= 9 && ((mshift - 5) & 3) == 0) {
+    // L = 32 16^k: a radix-32 first pass leaves radix-16 passes only (no radix-2
+    // pass at the end, 1/4 of the shared-memory traffic).  Butterfly j has inputs
+    // x_r at j + r L/32, zero for r >= 16; one thread computes its even outputs (the
+    // 16-point DFT of x_r), one its odd ones (of x_r w32^r).
+    const int half = tpr >> 1, h = lane >= half ? 1 : 0, j = lane - h * half, L32 = L >> 5;
+#pragma unroll
+    for (int r = 0; r < kElemsPerThread; ++r) {
+      const int z = j + r * L32;
+      v[r] = z < n ? __ldg(line + z) : make_float2(0.f, 0.f);
+    }
+    if (h) tw32_all(v);
+    dft_reg<16, false>(v);
+    float2* dst = X + 33 * j + h;
+#pragma unroll
+    for (int m = 0; m < 16; ++m) dst[2 * m] = v[m];
+    __syncthreads();
+    fft_rest<false, kLayoutFlat, 2, 5>(X, L, mshift, lane, tpr, tw, twstride, true, 5);
+  } else {
 #pragma unroll
     for (int r = 0; r < kElemsPerThread; ++r) {
       const int z = lane + r * tpr;
       v[r] = z < n ? __ldg(line + z) : make_float2(0.f, 0.f);
     }
     first_pass_regs<false>(X, v, lane);
+    __syncthreads();
+    fft_rest<false, kLayoutFlat>(X, L, mshift, lane, tpr, tw, twstride);
   }
-  __syncthreads();
-  fft_rest<false, kLayoutFlat>(X, L, mshift, lane, tpr, tw, twstride);
   if (!valid) return;
   float2* o = out + (size_t)row * (L / 2 + 2);
   for (int j = lane; j <= L / 2; j += tpr) {
@@ -336,7 +363,7 @@ cudaError_t launch_rows_fold(const float2* in, int n, float2* out, int L, int ro
   const int tpr = L / kElemsPerThread;
   const int threads = tpr > 128 ? tpr : 128;
   const int rpc = threads / tpr;
-  const size_t smem = (size_t)rpc * lateral_slot(L) * sizeof(float2);
+  const size_t smem = (size_t)rpc * rows_slot(L) * sizeof(float2);
   const cudaError_t e = cudaFuncSetAttribute(rows_fold_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   rows_fold_kernel<<<(rows + rpc - 1) / rpc, threads, smem, s>>>(in, n, out, L, mshift, rows, tw, twstride);

@@ -14,7 +14,7 @@ PAI_UNIT(9)
 
 size_t row_fft_region_bytes(int threads, int M) {
   const int tpr = M / kElemsPerThread;
-  return (size_t)(threads / tpr) * (size_t)row_slot_stride(M) * sizeof(float2);
+  return (size_t)(threads / tpr) * (size_t)row_slot_stride(M, 5) * sizeof(float2);
 }
 
 cudaError_t launch_row_forward(const RowLaunch& L, const WindowPoly& w, int threads, int ctas, size_t smem,

@@ -184,6 +184,7 @@ void fill_row_scalars(const pai_geometry& g, int M, int H, RowProblem& r) {
   r.rows = n1 * (n2 / 2 + 1);
   r.tpr = M / kElemsPerThread;
   r.slot = row_slot_stride(M);
+  r.slot32 = row_slot_stride(M, 5);
   r.mshift = 0;
   while ((1 << r.mshift) < M) ++r.mshift;
   r.nzshift = 0;
@@ -202,6 +203,7 @@ void fill_row_scalars(const pai_geometry& g, int M, int H, RowProblem& r) {
   const int tpu = pair ? 2 * r.tpr : r.tpr;
   band_layout(2 * B * 0.5 / g.dz, H, pair ? 4 : 3, tpu > 32 ? tpu / 32 : 1, (pair ? 2LL : 1LL) * r.slot, r.model_ps,
               r.model_slot);
+  r.model_dense = 2 * B <= 2.0 * g.nz * g.dz;
 }
 
 void twiddle_table(int TW, float2* tw) {

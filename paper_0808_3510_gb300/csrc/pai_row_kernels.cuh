@@ -40,7 +40,15 @@
 
 namespace pai {
 
-#define PADI(i) ((i) + ((i) >> 5))
+// Index of element i in the padded layout of a transform in shared memory: one
+// padding element every 2^PS.  With PS = 4 a radix-16 first pass (thread j
+// writes 16 j .. 16 j + 15) puts the 16 lanes of a half-warp on 16 different
+// banks (stride 17), with PS = 5 only on 8; after a radix-32 first pass
+// (33 j + q) PS = 5 is the one without conflicts.
+template <int PS = 4>
+__host__ __device__ __forceinline__ constexpr int padi(int i) {
+  return i + (i >> PS);
+}
 
 // Complex arithmetic on the packed two-lane FP32 instructions of sm_100+
 // (add/sub/mul/fma .rn.f32x2): one instruction per complex add, two per
@@ -173,7 +181,7 @@ __device__ __forceinline__ void dft_reg(float2 (&v)[R]) {
 }
 
 // Layouts of a row slot in shared memory.  Passes between the first and the
-// last keep one padding element every 32 (PADI) so strided butterfly accesses
+// last keep one padding element every 16 or 32 (padi) so strided butterfly accesses
 // do not collide in the banks.  The last pass of the forward transform writes
 // the spectrum unpadded and repeats its first 2*kMaxH values after index M
 // ("ghost cells"), so a node's 2H consecutive taps are plain consecutive
@@ -265,14 +273,13 @@ __device__ __forceinline__ void tw_apply(float2 (&v)[R], const TwBase<R>& t) {
   }
 }
 
-// Padded addresses without per-element shifts: for a multiple S of 32,
-// PADI(a + r S) = PADI(a) + r (S + S/32); and for a with a mod 32 < 16,
-// PADI(a + 16 r) = PADI(a) + 16 r + r/2 (r < 16).  Both hold for every pass
-// after the first radix-16 one (Ns = 16 or a multiple of 256), and for the
-// first pass (Ns = 1) PADI(16 j + r) = PADI(16 j) + r.
+// Padded addresses without per-element shifts: for a multiple S of 2^PS,
+// padi(a + r S) = padi(a) + r (S + S / 2^PS); for a with a mod 32 < 16,
+// padi<5>(a + 16 r) = padi<5>(a) + 16 r + r/2 (r < 16); and for a radix-16 first
+// pass (Ns = 1) padi(16 j + r) = padi(16 j) + r.
 // CHAIN_R: the smallest radix whose last pass derives its twiddles by
 // rotation (tw_shift); below it they come from the table.
-template <int R, bool INV, int OUT, int CHAIN_R = 2>
+template <int R, bool INV, int OUT, int CHAIN_R = 2, int PS = 4>
 __device__ __forceinline__ void fft_pass(float2* X, int M, int Ns, int lane, int tpr, const float2* __restrict__ tw,
                                          int twstride, bool active = true) {
   constexpr int NB = kElemsPerThread / R;
@@ -289,11 +296,11 @@ __device__ __forceinline__ void fft_pass(float2* X, int M, int Ns, int lane, int
   // several butterflies per thread and load after it to stay within registers
   if (active) {
     if (Ns > 1 && NB == 1) tw_load<R>(t[0], tw, (lane & (Ns - 1)) * tws);
-    if ((MR & 31) == 0) {
-      const int rs = MR + (MR >> 5);
+    if ((MR & ((1 << PS) - 1)) == 0) {
+      const int rs = MR + (MR >> PS);
 #pragma unroll
       for (int i = 0; i < NB; ++i) {
-        const float2* src = X + PADI(lane + i * tpr);
+        const float2* src = X + padi<PS>(lane + i * tpr);
 #pragma unroll
         for (int r = 0; r < R; ++r) v[i][r] = src[r * rs];
       }
@@ -302,7 +309,7 @@ __device__ __forceinline__ void fft_pass(float2* X, int M, int Ns, int lane, int
       for (int i = 0; i < NB; ++i) {
         const int j = lane + i * tpr;
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[i][r] = X[PADI(j + r * MR)];
+        for (int r = 0; r < R; ++r) v[i][r] = X[padi<PS>(j + r * MR)];
       }
     }
   }
@@ -322,12 +329,12 @@ __device__ __forceinline__ void fft_pass(float2* X, int M, int Ns, int lane, int
     dft_reg<R, INV>(v[i]);
     const int base = (j - k) * R + k;
     if (OUT == kLayoutPadded) {
-      float2* dst = X + PADI(base);
-      if (Ns == 16) {
+      float2* dst = X + padi<PS>(base);
+      if (PS == 5 && Ns == 16) {
 #pragma unroll
         for (int r = 0; r < R; ++r) dst[16 * r + (r >> 1)] = v[i][r];
-      } else if ((Ns & 31) == 0) {
-        const int ws = Ns + (Ns >> 5);
+      } else if (Ns > 1 && (Ns & ((1 << PS) - 1)) == 0) {
+        const int ws = Ns + (Ns >> PS);
 #pragma unroll
         for (int r = 0; r < R; ++r) dst[r * ws] = v[i][r];
       } else if (Ns == 1 && R == 16) {
@@ -335,7 +342,7 @@ __device__ __forceinline__ void fft_pass(float2* X, int M, int Ns, int lane, int
         for (int r = 0; r < R; ++r) dst[r] = v[i][r];
       } else {
 #pragma unroll
-        for (int r = 0; r < R; ++r) X[PADI(base + r * Ns)] = v[i][r];
+        for (int r = 0; r < R; ++r) X[padi<PS>(base + r * Ns)] = v[i][r];
       }
     } else {
       float2* dst = X + base;
@@ -400,7 +407,7 @@ __device__ __forceinline__ void fft_first_pass_from_global(float2* X, int M, int
     d8[7] = twq<1, true>(c8[7]);
     dft_reg<8, false>(c8);
     dft_reg<8, false>(d8);
-    float2* dst = X + PADI(lane * R);
+    float2* dst = X + padi<5>(lane * R);
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
       dst[2 * m] = c8[m];
@@ -422,10 +429,30 @@ __device__ __forceinline__ void fft_first_pass_from_global(float2* X, int M, int
     v[r] = a;
   }
   dft_reg<R, false>(v);
-  float2* dst = X + PADI(lane * R);
+  float2* dst = X + padi<5>(lane * R);
 #pragma unroll
   for (int r = 0; r < R; ++r) dst[r] = v[r];
   __syncthreads();
+}
+
+// v[r] *= e^{-2 pi i r / 32}, r = 0..15
+__device__ __forceinline__ void tw32_all(float2 (&v)[16]) {
+  v[1] = tw32<1, false>(v[1]);
+  v[2] = tw32<2, false>(v[2]);
+  v[3] = tw32<3, false>(v[3]);
+  v[4] = tw32<4, false>(v[4]);
+  v[5] = tw32<5, false>(v[5]);
+  v[6] = tw32<6, false>(v[6]);
+  v[7] = tw32<7, false>(v[7]);
+  v[8] = tw32<8, false>(v[8]);
+  // w32^r = -i w32^(r - 8)
+  v[9] = tw32<8, false>(tw32<1, false>(v[9]));
+  v[10] = tw32<8, false>(tw32<2, false>(v[10]));
+  v[11] = tw32<8, false>(tw32<3, false>(v[11]));
+  v[12] = tw32<8, false>(tw32<4, false>(v[12]));
+  v[13] = tw32<8, false>(tw32<5, false>(v[13]));
+  v[14] = tw32<8, false>(tw32<6, false>(v[14]));
+  v[15] = tw32<8, false>(tw32<7, false>(v[15]));
 }
 
 // First forward pass of radix 32 at oversampling 2 when M = 32 16^k: the
@@ -436,7 +463,7 @@ __device__ __forceinline__ void fft_first_pass_from_global(float2* X, int M, int
 // X[32 j + 2m] = sum_s z_s w16^{sm} with z_s = x_s + x_{s+16}, h = 1 the odd
 // ones with z_s = (x_s - x_{s+16}) w32^s, w_N = e^{-2 pi i/N}; of each pair
 // x_s, x_{s+16} one is padding (s < 8: x_{s+16}; s >= 8: x_s).  Both threads
-// load the butterfly's 16 samples.  Writes padded: PADI(32 j + q) = 33 j + q.
+// load the butterfly's 16 samples.  Writes padded: padi<5>(32 j + q) = 33 j + q.
 template <bool PAIRED>
 __device__ __forceinline__ void fft_first_pass32_from_global(float2* X, int M, int nt, int lane, int tpr,
                                                              const float2* __restrict__ src,
@@ -491,28 +518,28 @@ template <bool INV>
 __device__ __forceinline__ void first_pass_regs(float2* Z, float2 (&z)[kElemsPerThread], int x0) {
   dft_reg<kElemsPerThread, INV>(z);
 #pragma unroll
-  for (int r = 0; r < kElemsPerThread; ++r) Z[PADI(x0 * kElemsPerThread + r)] = z[r];
+  for (int r = 0; r < kElemsPerThread; ++r) Z[padi(x0 * kElemsPerThread + r)] = z[r];
 }
 
 // Remaining passes after a first pass of radix 2^ns_shift (16 or 32: Ns on
 // entry); the last pass writes layout OUT.
-template <bool INV, int OUT, int CHAIN_R = 2>
+template <bool INV, int OUT, int CHAIN_R = 2, int PS = 4>
 __device__ __forceinline__ void fft_rest(float2* X, int M, int mshift, int lane, int tpr, const float2* tw,
                                          int twstride, bool active = true, int ns_shift = 4) {
   int Ns = 1 << ns_shift;
   int rem = mshift - ns_shift;
   while (rem >= 4) {
     if (rem == 4) {
-      fft_pass<16, INV, OUT>(X, M, Ns, lane, tpr, tw, twstride, active);
+      fft_pass<16, INV, OUT, CHAIN_R, PS>(X, M, Ns, lane, tpr, tw, twstride, active);
       return;
     }
-    fft_pass<16, INV, kLayoutPadded>(X, M, Ns, lane, tpr, tw, twstride, active);
+    fft_pass<16, INV, kLayoutPadded, CHAIN_R, PS>(X, M, Ns, lane, tpr, tw, twstride, active);
     Ns <<= 4;
     rem -= 4;
   }
-  if (rem == 3) fft_pass<8, INV, OUT, CHAIN_R>(X, M, Ns, lane, tpr, tw, twstride, active);
-  else if (rem == 2) fft_pass<4, INV, OUT, CHAIN_R>(X, M, Ns, lane, tpr, tw, twstride, active);
-  else if (rem == 1) fft_pass<2, INV, OUT, CHAIN_R>(X, M, Ns, lane, tpr, tw, twstride, active);
+  if (rem == 3) fft_pass<8, INV, OUT, CHAIN_R, PS>(X, M, Ns, lane, tpr, tw, twstride, active);
+  else if (rem == 2) fft_pass<4, INV, OUT, CHAIN_R, PS>(X, M, Ns, lane, tpr, tw, twstride, active);
+  else if (rem == 1) fft_pass<2, INV, OUT, CHAIN_R, PS>(X, M, Ns, lane, tpr, tw, twstride, active);
 }
 
 // 16-byte shared-memory accesses by 32-bit address (the band grid below).
@@ -581,7 +608,7 @@ __device__ __forceinline__ void fft_first_pass_band(float2* X, int M, int lane, 
   }
   __syncthreads();
   dft_reg<R, true>(v);
-  float2* dst = X + PADI(lane * R);
+  float2* dst = X + padi(lane * R);
 #pragma unroll
   for (int r = 0; r < R; ++r) dst[r] = v[r];
   __syncthreads();
@@ -594,7 +621,7 @@ __device__ __forceinline__ void fft_first_pass_band(float2* X, int M, int lane, 
 // oversampling 2 only half of each butterfly's outputs are kept (and
 // computed): r < R/4 and r >= 3R/4, for R = 2 the first output of j < M/4 and
 // the second of the others.
-template <int R>
+template <int R, int PS>
 __device__ __forceinline__ void fft_last_crop(const float2* X, int M, int nt, int lane, int tpr,
                                               const float2* __restrict__ tw, int twstride, float2* dst,
                                               const float* __restrict__ prescale, float scale) {
@@ -604,7 +631,7 @@ __device__ __forceinline__ void fft_last_crop(const float2* X, int M, int nt, in
 #pragma unroll
   for (int i = 0; i < NB; ++i)
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[i][r] = X[PADI(lane + i * tpr + r * MR)];
+    for (int r = 0; r < R; ++r) v[i][r] = X[padi<PS>(lane + i * tpr + r * MR)];
   TwBase<R> t0, t;
   tw_load<R>(t0, tw, lane * twstride);
   const bool two = M == 2 * nt;
@@ -654,37 +681,40 @@ __device__ __forceinline__ void fft_last_crop(const float2* X, int M, int nt, in
 // kept, and only those 8 outputs are computed: with w = e^{+2 pi i/16},
 // A = inverse DFT8 of the even inputs and B of the odd,
 // Y[t] = A[t] + w^t B[t] (t = 0..3) and Y[t+8] = A[t] - w^t B[t] (t = 4..7).
-// BAND: the first pass reads the band grid.
+// BAND: the first pass reads the band grid.  (Otherwise one pad per 32, so
+// that the list spreads' rows and node lists fit in shared memory up to the
+// sizes they always did.)
 template <bool BAND>
 __device__ __forceinline__ void fft_inverse_crop(float2* X, int M, int mshift, int nt, int lane, int tpr,
                                                  const float2* __restrict__ tw, int twstride, float2* dst,
                                                  const float* __restrict__ prescale, float scale, bool valid,
                                                  const Band& band) {
+  constexpr int PS = BAND ? 4 : 5;
   if (BAND) fft_first_pass_band(X, M, lane, tpr, band);
-  else fft_pass<16, true, kLayoutPadded>(X, M, 1, lane, tpr, tw, twstride);
+  else fft_pass<16, true, kLayoutPadded, 2, PS>(X, M, 1, lane, tpr, tw, twstride);
   int Ns = 16;
   const int r0 = mshift & 3;
   while (Ns * 16 < M) {
-    fft_pass<16, true, kLayoutPadded>(X, M, Ns, lane, tpr, tw, twstride);
+    fft_pass<16, true, kLayoutPadded, 2, PS>(X, M, Ns, lane, tpr, tw, twstride);
     Ns <<= 4;
   }
   if (!valid) return;
   if (r0 != 0) {
-    if (r0 == 3) fft_last_crop<8>(X, M, nt, lane, tpr, tw, twstride, dst, prescale, scale);
-    else if (r0 == 2) fft_last_crop<4>(X, M, nt, lane, tpr, tw, twstride, dst, prescale, scale);
-    else fft_last_crop<2>(X, M, nt, lane, tpr, tw, twstride, dst, prescale, scale);
+    if (r0 == 3) fft_last_crop<8, PS>(X, M, nt, lane, tpr, tw, twstride, dst, prescale, scale);
+    else if (r0 == 2) fft_last_crop<4, PS>(X, M, nt, lane, tpr, tw, twstride, dst, prescale, scale);
+    else fft_last_crop<2, PS>(X, M, nt, lane, tpr, tw, twstride, dst, prescale, scale);
     return;
   }
   const int j = lane;
   float2 v[16];
-  if ((Ns & 31) == 0) {
-    const float2* src = X + PADI(j);
-    const int rs = Ns + (Ns >> 5);
+  if ((Ns & ((1 << PS) - 1)) == 0) {
+    const float2* src = X + padi<PS>(j);
+    const int rs = Ns + (Ns >> PS);
 #pragma unroll
     for (int r = 0; r < 16; ++r) v[r] = src[r * rs];
   } else {
 #pragma unroll
-    for (int r = 0; r < 16; ++r) v[r] = X[PADI(j + r * Ns)];
+    for (int r = 0; r < 16; ++r) v[r] = X[padi<PS>(j + r * Ns)];
   }
   if (Ns > 1) {
     TwBase<16> tb;
@@ -1083,7 +1113,7 @@ __global__ void __launch_bounds__(1024) row_forward_kernel(RowLaunch L, WindowPo
     const int lane = threadIdx.x - slot * tpr;
     const int row = wi.row0 + slot;
     const bool valid = row < P.rows;
-    float2* X = smem + slot * P.slot;
+    float2* X = smem + slot * P.slot32;
     // first pass straight from the lateral spectrum row (rows past the end read row 0, unused)
     const int srow = valid ? row : 0;
     const bool paired = PAIRED && P.paired != 0;
@@ -1101,7 +1131,9 @@ __global__ void __launch_bounds__(1024) row_forward_kernel(RowLaunch L, WindowPo
     }
     // (rotated twiddles only in radix-8 last passes: the register pressure of
     // the radix-2/4 ones costs this kernel more than the table loads)
-    fft_rest<false, kLayoutFlatGhost, 8>(X, M, P.mshift, lane, tpr, L.tw, L.Mmax >> P.mshift, true, r32 ? 5 : 4);
+    // (one pad per 32: a second instance of the passes for one pad per 16 cost this kernel more in registers than
+    // the first pass's two-way store conflicts: 54.0 against 51.8 us at M = 8192, 137.8 against 135.2 us at 256^3)
+    fft_rest<false, kLayoutFlatGhost, 8, 5>(X, M, P.mshift, lane, tpr, L.tw, L.Mmax >> P.mshift, true, r32 ? 5 : 4);
     if (valid) {
       if (!ZF) gather_row<H>(P, W, X, row, lane);
       else gather_row_z<H>(P, W, X, P.fh + (size_t)row * P.nz, row, lane);
@@ -1365,6 +1397,53 @@ __device__ __forceinline__ void band_spread(const WindowPoly& W, const BandTaps<
   }
 }
 
+// Spreads two neighbouring nodes A and B per lane, d = 0, 1 or 2 cells apart:
+// their 2H + 2 cells take both nodes' terms in one read and write each, B's
+// weights shifted by d, so a node costs H + 1 accesses instead of 2H, and lanes
+// share a cell only where four nodes do.  Runs sum by shuffles.
+template <int H, bool WIDE>
+__device__ __forceinline__ void band_spread2(const WindowPoly& W, const BandTaps<WIDE>& tp, int j0, float fa,
+                                             const Cell<WIDE>& qa, bool act, int gw, int d, float fb,
+                                             const Cell<WIDE>& qb) {
+  const float za = fa - 0.5f, za2 = za * za, zb = fb - 0.5f, zb2 = zb * zb;
+  const Runs r = find_runs(j0, act, gw);
+  const int l32 = threadIdx.x & 31;
+  // cell u: wa A + (b0, b1 or b2) B, the three candidates for d = 0, 1, 2
+  auto cell = [&](int u, float wa, float b0, float b1, float b2) {
+    const float wb = d == 0 ? b0 : d == 1 ? b1 : b2;
+    const unsigned a = tp.at(u);
+    if (r.maxrun <= 1) {
+      if (act) cell_store<WIDE>(a, cell_axpy<WIDE>(wb, qb, cell_axpy<WIDE>(wa, qa, cell_load<WIDE>(a))));
+    } else {
+      Cell<WIDE> v = cell_axpy<WIDE>(wb, qb, cell_axpy<WIDE>(wa, qa, cell_zero<WIDE>()));
+      for (int k = 1; k < r.maxrun; k <<= 1) {
+        const Cell<WIDE> t = cell_shfl_down<WIDE>(v, k);
+        if (l32 + k <= r.last) v = cell_add<WIDE>(v, t);
+      }
+      if (r.head) cell_store<WIDE>(a, cell_add<WIDE>(cell_load<WIDE>(a), v));
+    }
+    __syncwarp();
+  };
+  // from both ends inwards: lower and upper weights of this and the last two pairs
+  float l1 = 0.f, l2 = 0.f, u1 = 0.f, u2 = 0.f, ua1 = 0.f, ua2 = 0.f;
+#pragma unroll
+  for (int p = 0; p < H; ++p) {
+    float la, ha, lb, hb;
+    tap_pair<H>(W, p, za, za2, la, ha);
+    tap_pair<H>(W, p, zb, zb2, lb, hb);
+    cell(p, la, lb, l1, l2);
+    cell(2 * H + 1 - p, ua2, u2, u1, hb);
+    l2 = l1;
+    l1 = lb;
+    u2 = u1;
+    u1 = hb;
+    ua2 = ua1;
+    ua1 = ha;
+  }
+  cell(H, ua1, u1, l1, l2);
+  cell(H + 1, ua2, u2, u1, l1);
+}
+
 // A row's (or unit's) sorted nodes divided over its warps, and the part of the
 // band each warp adds to.  Cells at or below the predecessor's last cell go to
 // the warp's own spill of kSpill cells and are merged after a barrier; all
@@ -1606,26 +1685,52 @@ __global__ void __launch_bounds__(1024) row_model_kernel(RowLaunch L, WindowPoly
       node(i, j0, fr);
       return j0;
     });
-    const int cn = __reduce_max_sync(0xffffffffu, (unsigned)(part.n1 - part.n0));
-    for (int c0 = 0; c0 < cn; c0 += part.gw) {
-      const int i = part.n0 + c0 + part.l;
-      const bool act = i < part.n1;
-      int j0 = 0;
-      float fr = 0.5f;
-      Cell<PAIR> q = cell_zero<PAIR>();
-      if (act) {
-        const float2 ya = __ldg(za + i);
-        if constexpr (PAIR) {
-          const float2 yb = row_b >= 0 ? __ldg(zb + i) : make_float2(0.f, 0.f);
-          q.v = make_float4(P.wscale * ya.x, P.wscale * ya.y, P.wscale * yb.x, P.wscale * yb.y);
-        } else {
-          q.v = make_float2(P.wscale * ya.x, P.wscale * ya.y);
-        }
-        node(i, j0, fr);
+    auto value = [&](int i) {
+      const float2 ya = __ldg(za + i);
+      if constexpr (PAIR) {
+        const float2 yb = row_b >= 0 ? __ldg(zb + i) : make_float2(0.f, 0.f);
+        return Cell<true>{make_float4(P.wscale * ya.x, P.wscale * ya.y, P.wscale * yb.x, P.wscale * yb.y)};
+      } else {
+        return Cell<false>{make_float2(P.wscale * ya.x, P.wscale * ya.y)};
       }
-      const int c = j0 - H + 1;
-      const BandTaps<PAIR> tp(band, c - band.lo, part.spill_w + ((c - part.lo_w) << kShift), part.hi_prev + 1 - c);
-      band_spread<H, PAIR>(W, tp, j0, fr, q, act, part.gw);
+    };
+    const int cn = __reduce_max_sync(0xffffffffu, (unsigned)(part.n1 - part.n0));
+    for (int c0 = 0; c0 < cn;) {
+      // two nodes per lane while there are enough and they are at most two cells apart
+      const bool two = P.model_dense && cn - c0 > part.gw;
+      const int step = two ? 2 : 1;
+      const int i = part.n0 + c0 + step * part.l;
+      c0 += step * part.gw;
+      const bool act = i < part.n1;
+      int j0 = 0, jb = 0;
+      float fr = 0.5f, fb = 0.5f;
+      Cell<PAIR> q = cell_zero<PAIR>(), qb = q;
+      if (act) {
+        q = value(i);
+        node(i, j0, fr);
+        jb = j0;
+      }
+      if (two) {
+        const bool actb = i + 1 < part.n1;
+        if (actb) {
+          qb = value(i + 1);
+          node(i + 1, jb, fb);
+        }
+        const int prev = __shfl_up_sync(0xffffffffu, jb, 1);
+        // (rounding may move a node by a cell: then one at a time)
+        if (__all_sync(0xffffffffu, !act || (jb >= j0 && jb <= j0 + 2 && (part.l == 0 || prev <= j0)))) {
+          const int c = j0 - H + 1;
+          const BandTaps<PAIR> tp(band, c - band.lo, part.spill_w + ((c - part.lo_w) << kShift), part.hi_prev + 1 - c);
+          band_spread2<H, PAIR>(W, tp, j0, fr, q, act, part.gw, jb - j0, fb, qb);
+          continue;
+        }
+      }
+      for (int k = 0; k < step; ++k) {
+        const bool on = k == 0 ? act : i + 1 < part.n1;
+        const int j = k == 0 ? j0 : jb, c = j - H + 1;
+        const BandTaps<PAIR> tp(band, c - band.lo, part.spill_w + ((c - part.lo_w) << kShift), part.hi_prev + 1 - c);
+        band_spread<H, PAIR>(W, tp, j, k == 0 ? fr : fb, k == 0 ? q : qb, on, part.gw);
+      }
     }
     __syncthreads();
     band_end<H, PAIR>(part, band, lane_u, tpu, 2 * M);
@@ -1683,7 +1788,7 @@ __global__ void __launch_bounds__(1024) row_adjoint_kernel(RowLaunch L, WindowPo
     const int lane = threadIdx.x - slot * tpr;
     const int row = wi.row0 + slot;
     const bool valid = row < P.rows;
-    float2* X = smem + slot * P.slot;
+    float2* X = smem + slot * P.slot32;
     float4* N = nodes_all + slot * (P.nz + 2);
     const int nzh = P.nz >> 1;
     RowGeom rg;
@@ -1813,7 +1918,7 @@ __global__ void __launch_bounds__(1024) row_adjoint_kernel(RowLaunch L, WindowPo
       // grid, no tap phases (summation order, hence the last bits, may vary
       // from run to run)
       const bool interp = H == 2 && P.method >= PAI_METHOD_LINEAR;
-      for (int g = lane; g < M; g += tpr) X[PADI(g)] = make_float2(0.f, 0.f);
+      for (int g = lane; g < M; g += tpr) X[padi<5>(g)] = make_float2(0.f, 0.f);
       __syncthreads();
       for (int i = lane; i < nn; i += tpr) {
         const float4 nd = N[i];
@@ -1834,8 +1939,8 @@ __global__ void __launch_bounds__(1024) row_adjoint_kernel(RowLaunch L, WindowPo
               wh = interp_tap_weight(P.method, 2 * H - 1 - p, nd.y);
             }
           }
-          float2* cl = X + PADI((j0 + p - H + 1) & mask);
-          float2* ch = X + PADI((j0 + H - p) & mask);
+          float2* cl = X + padi<5>((j0 + p - H + 1) & mask);
+          float2* ch = X + padi<5>((j0 + H - p) & mask);
           atomicAdd(&cl->x, wl * nd.z);
           atomicAdd(&cl->y, wl * nd.w);
           atomicAdd(&ch->x, wh * nd.z);
@@ -1848,7 +1953,7 @@ __global__ void __launch_bounds__(1024) row_adjoint_kernel(RowLaunch L, WindowPo
       // sums the run's weighted terms for every tap and adds each sum with one
       // atomic, so clusters of nodes on few cells cost few atomics
       const bool interp = H == 2 && P.method >= PAI_METHOD_LINEAR;
-      for (int g = lane; g < M; g += tpr) X[PADI(g)] = make_float2(0.f, 0.f);
+      for (int g = lane; g < M; g += tpr) X[padi<5>(g)] = make_float2(0.f, 0.f);
       __syncthreads();
       for (int i = lane; i < nn; i += tpr) {
         const int j0 = __float_as_int(N[i].x);
@@ -1879,8 +1984,8 @@ __global__ void __launch_bounds__(1024) row_adjoint_kernel(RowLaunch L, WindowPo
             hx = fmaf(wh, nd.z, hx);
             hy = fmaf(wh, nd.w, hy);
           }
-          float2* cl = X + PADI((j0 + p - H + 1) & mask);
-          float2* ch = X + PADI((j0 + H - p) & mask);
+          float2* cl = X + padi<5>((j0 + p - H + 1) & mask);
+          float2* ch = X + padi<5>((j0 + H - p) & mask);
           atomicAdd(&cl->x, lx);
           atomicAdd(&cl->y, ly);
           atomicAdd(&ch->x, hx);
@@ -1891,7 +1996,7 @@ __global__ void __launch_bounds__(1024) row_adjoint_kernel(RowLaunch L, WindowPo
     } else {
       const int CH = L.chunk;  // <= tpr
       const bool interp = H == 2 && P.method >= PAI_METHOD_LINEAR;
-      for (int g = lane; g < M; g += tpr) X[PADI(g)] = make_float2(0.f, 0.f);
+      for (int g = lane; g < M; g += tpr) X[padi<5>(g)] = make_float2(0.f, 0.f);
       const int list_max = (P.nz >> 1) + (P.qmode ? 1 : 0);  // nodes per sign list, at most
       const int half_chunks = (list_max + CH - 1) / CH;         // uniform over the CTA's slots
       for (int c = 0; c < 2 * half_chunks; ++c) {
@@ -1949,7 +2054,7 @@ __global__ void __launch_bounds__(1024) row_adjoint_kernel(RowLaunch L, WindowPo
                 sx = fmaf(w, nd.z, sx);
                 sy = fmaf(w, nd.w, sy);
               }
-              const int gi = PADI((j0 + t - H + 1) & mask);
+              const int gi = padi<5>((j0 + t - H + 1) & mask);
               float2 x = X[gi];
               x.x += sx;
               x.y += sy;
@@ -1963,7 +2068,7 @@ __global__ void __launch_bounds__(1024) row_adjoint_kernel(RowLaunch L, WindowPo
     if constexpr (H == 2) {
       // interpolation methods: the grid cells' phases e^{+i pi nu_j}
       if (valid && P.method >= PAI_METHOD_LINEAR)
-        for (int g = lane; g < M; g += tpr) X[PADI(g)] = cmul(X[PADI(g)], node_phase(g, 0.0f, nt, M, P.nt_over_M));
+        for (int g = lane; g < M; g += tpr) X[padi<5>(g)] = cmul(X[padi<5>(g)], node_phase(g, 0.0f, nt, M, P.nt_over_M));
     }
     __syncthreads();
     const float scale = (valid && !ZF && rg.mirror) ? 0.5f : 1.0f;
