@@ -86,6 +86,19 @@ struct pai_plan_s {
   bool zf = false;      // forward: every stage by the library's kernels (depth-row layout)
   bool zf_adj = false;  // adjoint: the same choice, tuned separately
   size_t smem_fwd = 0, smem_adj = 0;
+  bool pdl() const { return nbranch <= 1; }  // one stream: kernels launch as programmatic dependents
+  // Whether repeated calls replay a graph.  A single problem on the library's
+  // kernels is four to six launches: as programmatic dependents on the caller's
+  // stream they follow each other (and the previous call) closer than graph
+  // replays do (128^3: 53.8 us a pass against 60.7 with a graph; 2048x4096: 97.7
+  // and 104.2), unless the problem is so small that the launches themselves take
+  // longer than the kernels (128x256: 20.9 and 17.2 us; the two meet near 20 us a
+  // pass, about a million samples and voxels).  Calls of many cuFFT launches and
+  // of batches replay a graph.
+  bool graphed(bool adjoint) const {
+    if (!use_graph) return false;
+    return probs.size() > 1 || !(adjoint ? zf_adj : zf) || data_total + img_total < ((size_t)1 << 20);
+  }
   WindowPoly poly{};
   double beta = 0, pred_err = 0, fit_err = 0;
   size_t data_total = 0, img_total = 0;
@@ -140,6 +153,8 @@ struct pai_plan_s {
   int fft_made = 0;
   size_t items_fwd_bytes = 0, items_adj_bytes = 0;
   std::vector<GraphEntry> graphs;
+  GraphEntry seen[8];  // buffers of the last calls launched directly
+  unsigned seen_next = 0;
   long long own_kernels = 0, fft_execs = 0;
   int own_kernels_per_call = 0, fft_per_call = 0;
   int own_kernels_per_adj = 0, fft_per_adj = 0;
@@ -361,6 +376,7 @@ RowLaunch make_launch(pai_plan_s* P, bool adjoint) {
     L.model_pair = P->probs[0].g.dim == 3 ? 1 : 0;
   }
   L.paired = !adjoint && P->any_paired ? 1 : 0;
+  L.pdl = P->pdl();
   return L;
 }
 
@@ -387,18 +403,18 @@ pai_status enqueue_row(pai_plan_s* P, bool adjoint, cudaStream_t s, int threads,
 // along x.  The adjoint uses the same transform on the image (C = nz).
 pai_status own_lateral_fwd(pai_plan_s* P, const ProblemHost& p, const float* in, float2* out, int C, cudaStream_t s) {
   const pai_geometry& g = p.g;
-  if (g.dim == 2) return cuda_status(launch_lateral_r2c(in, out, g.nx, C, 1, P->d_tw, P->TW / g.nx, s));
-  PAI_CUDA(launch_lateral_r2c(in, out, g.ny, C, g.nx, P->d_tw, P->TW / g.ny, s));
-  return cuda_status(launch_lateral_c2c(out, out, g.nx, (g.ny / 2 + 1) * C, 1, false, P->d_tw, P->TW / g.nx, s));
+  if (g.dim == 2) return cuda_status(launch_lateral_r2c(in, out, g.nx, C, 1, P->d_tw, P->TW / g.nx, s, P->pdl()));
+  PAI_CUDA(launch_lateral_r2c(in, out, g.ny, C, g.nx, P->d_tw, P->TW / g.ny, s, P->pdl()));
+  return cuda_status(launch_lateral_c2c(out, out, g.nx, (g.ny / 2 + 1) * C, 1, false, P->d_tw, P->TW / g.nx, s, P->pdl()));
 }
 
 // Lateral inverse (Hermitian C2R) of complex rows in[row][c] into the real
 // array out[x][(y)][c]; 3-D runs the C2C along x in place on `in` first.
 pai_status own_lateral_inv(pai_plan_s* P, const ProblemHost& p, float2* in, float* out, int C, cudaStream_t s) {
   const pai_geometry& g = p.g;
-  if (g.dim == 2) return cuda_status(launch_lateral_c2r(in, out, g.nx, C, 1, P->d_tw, P->TW / g.nx, s));
-  PAI_CUDA(launch_lateral_c2c(in, in, g.nx, (g.ny / 2 + 1) * C, 1, true, P->d_tw, P->TW / g.nx, s));
-  return cuda_status(launch_lateral_c2r(in, out, g.ny, C, g.nx, P->d_tw, P->TW / g.ny, s));
+  if (g.dim == 2) return cuda_status(launch_lateral_c2r(in, out, g.nx, C, 1, P->d_tw, P->TW / g.nx, s, P->pdl()));
+  PAI_CUDA(launch_lateral_c2c(in, in, g.nx, (g.ny / 2 + 1) * C, 1, true, P->d_tw, P->TW / g.nx, s, P->pdl()));
+  return cuda_status(launch_lateral_c2r(in, out, g.ny, C, g.nx, P->d_tw, P->TW / g.ny, s, P->pdl()));
 }
 
 // Stage (a) of the forward operator for problem p.
@@ -414,7 +430,7 @@ pai_status enqueue_lateral(pai_plan_s* P, const ProblemHost& p, const float* d_p
 // depth FFT of every row, then the lateral C2R.
 pai_status enqueue_inverse(pai_plan_s* P, const ProblemHost& p, float* d_f, cudaStream_t s) {
   if (P->zf) {
-    PAI_CUDA(launch_rows_c2c(P->d_fh + p.fh_off, p.g.nz, p.rows, true, P->d_tw, P->TW / p.g.nz, s));
+    PAI_CUDA(launch_rows_c2c(P->d_fh + p.fh_off, p.g.nz, p.rows, true, P->d_tw, P->TW / p.g.nz, s, P->pdl()));
     return own_lateral_inv(P, p, P->d_fh + p.fh_off, d_f + p.img_off, p.g.nz, s);
   }
   return fft_status(cufftExecC2R(p.img_c2r, (cufftComplex*)(P->d_fh + p.fh_off), d_f + p.img_off));
@@ -430,20 +446,20 @@ pai_status enqueue_model_first(pai_plan_s* P, const ProblemHost& p, const float*
   const pai_geometry &b = p.g, &gi = P->qimg;
   const float2* tw = P->d_tw;
   if (b.dim == 2) {
-    PAI_CUDA(launch_lateral_r2c(d_f, P->d_pt, b.nx, gi.nz, 1, tw, P->TW / b.nx, s, gi.nx));
+    PAI_CUDA(launch_lateral_r2c(d_f, P->d_pt, b.nx, gi.nz, 1, tw, P->TW / b.nx, s, P->pdl(), gi.nx));
   } else {
-    PAI_CUDA(launch_lateral_r2c(d_f, P->d_fh, b.ny, gi.nz, gi.nx, tw, P->TW / b.ny, s, gi.ny));
-    PAI_CUDA(launch_lateral_c2c(P->d_fh, P->d_pt, b.nx, (b.ny / 2 + 1) * gi.nz, 1, false, tw, P->TW / b.nx, s, gi.nx));
+    PAI_CUDA(launch_lateral_r2c(d_f, P->d_fh, b.ny, gi.nz, gi.nx, tw, P->TW / b.ny, s, P->pdl(), gi.ny));
+    PAI_CUDA(launch_lateral_c2c(P->d_fh, P->d_pt, b.nx, (b.ny / 2 + 1) * gi.nz, 1, false, tw, P->TW / b.nx, s, P->pdl(), gi.nx));
   }
-  return cuda_status(launch_rows_fold(P->d_pt, gi.nz, P->d_fh, b.nz, p.rows, tw, P->TW / b.nz, s));
+  return cuda_status(launch_rows_fold(P->d_pt, gi.nz, P->d_fh, b.nz, p.rows, tw, P->TW / b.nz, s, P->pdl()));
 }
 
 pai_status enqueue_model_last(pai_plan_s* P, const ProblemHost& p, float* d_p, cudaStream_t s) {
   const pai_geometry &b = p.g, &gi = P->qimg;
   const float2* tw = P->d_tw;
-  if (b.dim == 2) return cuda_status(launch_lateral_c2r(P->d_pt, d_p, b.nx, b.nt, 1, tw, P->TW / b.nx, s, gi.nx));
-  PAI_CUDA(launch_lateral_c2c(P->d_pt, P->d_pt, b.nx, (b.ny / 2 + 1) * b.nt, 1, true, tw, P->TW / b.nx, s, gi.nx));
-  return cuda_status(launch_lateral_c2r(P->d_pt, d_p, b.ny, b.nt, gi.nx, tw, P->TW / b.ny, s, gi.ny));
+  if (b.dim == 2) return cuda_status(launch_lateral_c2r(P->d_pt, d_p, b.nx, b.nt, 1, tw, P->TW / b.nx, s, P->pdl(), gi.nx));
+  PAI_CUDA(launch_lateral_c2c(P->d_pt, P->d_pt, b.nx, (b.ny / 2 + 1) * b.nt, 1, true, tw, P->TW / b.nx, s, P->pdl(), gi.nx));
+  return cuda_status(launch_lateral_c2r(P->d_pt, d_p, b.ny, b.nt, gi.nx, tw, P->TW / b.ny, s, P->pdl(), gi.ny));
 }
 
 // First and last stages of the adjoint for problem p.
@@ -451,7 +467,7 @@ pai_status enqueue_adj_first(pai_plan_s* P, const ProblemHost& p, const float* d
   if (P->qmode) return enqueue_model_first(P, p, d_h, s);
   if (P->zf_adj) {
     PAI_TRY(own_lateral_fwd(P, p, d_h + p.img_off, P->d_fh + p.fh_off, p.g.nz, s));
-    return cuda_status(launch_rows_c2c(P->d_fh + p.fh_off, p.g.nz, p.rows, false, P->d_tw, P->TW / p.g.nz, s));
+    return cuda_status(launch_rows_c2c(P->d_fh + p.fh_off, p.g.nz, p.rows, false, P->d_tw, P->TW / p.g.nz, s, P->pdl()));
   }
   return fft_status(cufftExecR2C(p.img_r2c, const_cast<float*>(d_h) + p.img_off, (cufftComplex*)(P->d_fh + p.fh_off)));
 }
@@ -525,15 +541,30 @@ pai_status enqueue_adjoint(pai_plan_s* P, const float* d_h, float* d_pbar, cudaS
 pai_status run(pai_plan_s* P, const void* in, void* out, bool adjoint) {
   int prev = 0;
   cudaGetDevice(&prev);
-  if (prev != P->device) cudaSetDevice(P->device);
+  // also when it is the current device already: in a thread that has made no
+  // CUDA call yet (autograd's backward threads) this makes its context current,
+  // which a direct cuFFT execution needs
+  cudaSetDevice(P->device);
   pai_status st = PAI_OK;
-  if (!P->use_graph) {
+  GraphEntry* hit = nullptr;
+  bool direct = !P->graphed(adjoint);
+  if (!direct) {
+    for (auto& ge : P->graphs)
+      if (ge.in == in && ge.out == out && ge.adjoint == adjoint) hit = &ge;
+    if (!hit) {
+      // buffers not seen lately: launch directly (a capture costs several
+      // passes); a second call with them captures
+      const GraphEntry now{in, out, adjoint, nullptr};
+      direct = true;
+      for (auto& ge : P->seen)
+        if (ge.in == in && ge.out == out && ge.adjoint == adjoint) direct = false;
+      if (direct) P->seen[P->seen_next++ % 8] = now;
+    }
+  }
+  if (direct) {
     st = adjoint ? enqueue_adjoint(P, (const float*)in, (float*)out, P->stream)
                  : enqueue_forward(P, (const float*)in, (float*)out, P->stream, false);
   } else {
-    GraphEntry* hit = nullptr;
-    for (auto& ge : P->graphs)
-      if (ge.in == in && ge.out == out && ge.adjoint == adjoint) hit = &ge;
     if (!hit) {
       // capture on the private stream (the caller's stream may be the legacy default stream)
       st = set_fft_streams(P, P->cap_stream);
@@ -1660,7 +1691,7 @@ pai_status pai_get_info(pai_plan_t plan, pai_plan_info* info) {
   info->rows = plan->rows_total;
   info->nodes = plan->nodes;
   info->workspace_bytes = plan->ws_bytes;
-  info->uses_graph = plan->use_graph ? 1 : 0;
+  info->uses_graph = plan->graphed(false) || plan->graphed(true) ? 1 : 0;
   info->library_ffts = (plan->zf ? 1 : 0) | (plan->zf_adj ? 2 : 0);
   return PAI_OK;
 }

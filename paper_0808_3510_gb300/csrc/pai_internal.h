@@ -5,11 +5,47 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
 #include <vector>
 
 #include "../../include/pai.h"
 
 namespace pai {
+
+// Launches a kernel; pdl: as a programmatic dependent of the stream's previous
+// kernel, so that its CTAs are set up while that one drains (every kernel here
+// begins with pdl_wait(), which returns when the previous kernel is complete
+// and its writes are visible).  Not for launches that join several streams.
+template <typename... P, typename... A>
+inline cudaError_t launch_kernel(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool pdl,
+                                 A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&c, k, P(args)...);
+}
+// Allows `smem` bytes of dynamic shared memory; up to 48 KB (with the static part) need no call.
+template <typename K>
+inline cudaError_t allow_smem(K* kernel, size_t smem) {
+  if (smem <= 47 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+#ifdef __CUDACC__
+// First statement of a kernel: waits for the previous one.  (The next kernel's
+// CTAs come when this one's leave; letting them in earlier,
+// griddepcontrol.launch_dependents, had them hold shared memory while they
+// waited: 128^3 65.7 against 60.7 us, 128x256 18.7 against 17.2 us.)
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+#endif
 
 // Largest half tap count supported by the row kernels: taps per node = 2H <= 24.
 constexpr int kMaxH = 12;
@@ -104,6 +140,7 @@ struct RowLaunch {
                                // into band grids (deterministic; windowed methods; not qmode), 4 the
                                // forward-model row kernel (deterministic; qmode only)
   int model_pair;              // spread mode 4: units of two rows (3-D)
+  bool pdl;                    // launch as a programmatic dependent (launch_kernel)
   int paired;                  // forward: some problem is in the paired layout (RowProblem::paired)
 };
 
@@ -187,18 +224,18 @@ bool lateral_supported(int L, int C);
 // n (0: L): only the first n of the L points of the axis exist on the side named real (c2c: on the input of the
 // forward, the output of the inverse transform): A[outer][n][C]; the others are zeros (input) or not wanted (output).
 cudaError_t launch_lateral_r2c(const float* in, float2* out, int L, int C, int outer, const float2* tw, int twstride,
-                               cudaStream_t s, int n = 0);
+                               cudaStream_t s, bool pdl, int n = 0);
 cudaError_t launch_lateral_c2r(const float2* in, float* out, int L, int C, int outer, const float2* tw, int twstride,
-                               cudaStream_t s, int n = 0);
+                               cudaStream_t s, bool pdl, int n = 0);
 cudaError_t launch_lateral_c2c(const float2* in, float2* out, int L, int C, int outer, bool inverse, const float2* tw,
-                               int twstride, cudaStream_t s, int n = 0);
+                               int twstride, cudaStream_t s, bool pdl, int n = 0);
 // In-place FFT of `rows` contiguous complex lines of power-of-two length L (32 <= L <= 16384).
 cudaError_t launch_rows_c2c(float2* data, int L, int rows, bool inverse, const float2* tw, int twstride,
-                            cudaStream_t s);
+                            cudaStream_t s, bool pdl);
 // Forward FFT of `rows` lines in[row][n] zero-padded to length L, folded: out[row][j] = F[j] + F[L - j] for
 // 0 < j < L/2, F[0] and F[L/2] alone (j = 0..L/2; out lines are L/2 + 2 values apart).
 cudaError_t launch_rows_fold(const float2* in, int n, float2* out, int L, int rows, const float2* tw, int twstride,
-                             cudaStream_t s);
+                             cudaStream_t s, bool pdl);
 // kind: 0 forward row kernel, 1 adjoint row kernel, 2 adjoint row kernel with the pair spread, 3 forward row
 // kernel for launches with problems in the paired layout, 4 forward-model row kernel, 5 the same in units of two rows
 int row_kernel_max_ctas_per_sm(int kind, int threads, size_t smem, int H, bool zf = false);

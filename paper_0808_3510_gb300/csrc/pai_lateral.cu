@@ -69,6 +69,7 @@ __global__ void __launch_bounds__(1024) lateral_kernel(const void* vin, void* vo
   const int c0 = blockIdx.x * CPT;
   const long long ob = blockIdx.y;
   float2* Z = smem + f * S;
+  pdl_wait();
 
   // ---- load -------------------------------------------------------------
   if (KIND == kLatR2C) {
@@ -186,10 +187,10 @@ bool lateral_supported(int L, int C) {
 
 template <int KIND, int FP, bool PRUNED>
 static cudaError_t lat_launch(const void* in, void* out, int L, int C, int outer, long long in_outer,
-                              long long out_outer, const float2* tw, int twstride, cudaStream_t s, int n) {
+                              long long out_outer, const float2* tw, int twstride, cudaStream_t s, bool pdl, int n) {
   const size_t smem = lateral_smem_bytes(L);
   cudaError_t e =
-      cudaFuncSetAttribute(lateral_kernel<KIND, FP, PRUNED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      allow_smem(lateral_kernel<KIND, FP, PRUNED>, smem);
   if (e != cudaSuccess) return e;
   int mshift = 0;
   while ((1 << mshift) < L) ++mshift;
@@ -198,50 +199,49 @@ static cudaError_t lat_launch(const void* in, void* out, int L, int C, int outer
   dim3 grid((C + CPT - 1) / CPT, outer);
   const void* real = KIND == kLatR2C ? in : out;
   const int pairs = (reinterpret_cast<uintptr_t>(real) & 7) == 0;
-  lateral_kernel<KIND, FP, PRUNED>
-      <<<grid, threads, smem, s>>>(in, out, L, mshift, C, in_outer, out_outer, tw, twstride, n, pairs);
-  return cudaGetLastError();
+  return launch_kernel(lateral_kernel<KIND, FP, PRUNED>, grid, dim3(threads), smem, s, pdl, in, out, L, mshift, C,
+                       in_outer, out_outer, tw, twstride, n, pairs);
 }
 
 // in_full / out_full: outer strides for L (complex kinds) or L/2 + 1 points; the pruned side has n.
 template <int KIND, bool PRUNED>
 static cudaError_t lat_dispatch(const void* in, void* out, int L, int C, int outer, const float2* tw, int twstride,
-                                cudaStream_t s, int n) {
+                                cudaStream_t s, bool pdl, int n) {
   const long long full = (long long)L * C, half = (long long)(L / 2 + 1) * C, part = (long long)n * C;
   const long long io = KIND == kLatC2R ? half : KIND == kLatC2CInv ? full : part;
   const long long oo = KIND == kLatR2C ? half : KIND == kLatC2C ? full : part;
   switch (lateral_slots_per_cta(L)) {
-    case 8: return lat_launch<KIND, 8, PRUNED>(in, out, L, C, outer, io, oo, tw, twstride, s, n);
-    case 4: return lat_launch<KIND, 4, PRUNED>(in, out, L, C, outer, io, oo, tw, twstride, s, n);
-    case 2: return lat_launch<KIND, 2, PRUNED>(in, out, L, C, outer, io, oo, tw, twstride, s, n);
-    default: return lat_launch<KIND, 1, PRUNED>(in, out, L, C, outer, io, oo, tw, twstride, s, n);
+    case 8: return lat_launch<KIND, 8, PRUNED>(in, out, L, C, outer, io, oo, tw, twstride, s, pdl, n);
+    case 4: return lat_launch<KIND, 4, PRUNED>(in, out, L, C, outer, io, oo, tw, twstride, s, pdl, n);
+    case 2: return lat_launch<KIND, 2, PRUNED>(in, out, L, C, outer, io, oo, tw, twstride, s, pdl, n);
+    default: return lat_launch<KIND, 1, PRUNED>(in, out, L, C, outer, io, oo, tw, twstride, s, pdl, n);
   }
 }
 
 template <int KIND>
 static cudaError_t lat_any(const void* in, void* out, int L, int C, int outer, const float2* tw, int twstride,
-                           cudaStream_t s, int n) {
-  if (n > 0 && n < L) return lat_dispatch<KIND, true>(in, out, L, C, outer, tw, twstride, s, n);
-  return lat_dispatch<KIND, false>(in, out, L, C, outer, tw, twstride, s, L);
+                           cudaStream_t s, bool pdl, int n) {
+  if (n > 0 && n < L) return lat_dispatch<KIND, true>(in, out, L, C, outer, tw, twstride, s, pdl, n);
+  return lat_dispatch<KIND, false>(in, out, L, C, outer, tw, twstride, s, pdl, L);
 }
 
 // out[o][k][c] = sum_x e^{-2 pi i k x / L} in[o][x][c], k = 0..L/2.
 cudaError_t launch_lateral_r2c(const float* in, float2* out, int L, int C, int outer, const float2* tw, int twstride,
-                               cudaStream_t s, int n) {
-  return lat_any<kLatR2C>(in, out, L, C, outer, tw, twstride, s, n);
+                               cudaStream_t s, bool pdl, int n) {
+  return lat_any<kLatR2C>(in, out, L, C, outer, tw, twstride, s, pdl, n);
 }
 
 // out[o][x][c] = sum over the Hermitian extension of in[o][k][c] of e^{+2 pi i k x / L} (unnormalised C2R).
 cudaError_t launch_lateral_c2r(const float2* in, float* out, int L, int C, int outer, const float2* tw, int twstride,
-                               cudaStream_t s, int n) {
-  return lat_any<kLatC2R>(in, out, L, C, outer, tw, twstride, s, n);
+                               cudaStream_t s, bool pdl, int n) {
+  return lat_any<kLatC2R>(in, out, L, C, outer, tw, twstride, s, pdl, n);
 }
 
 // out[o][k][c] = sum_x e^{-+2 pi i k x / L} in[o][x][c]; in place allowed when not pruned (each CTA owns its columns).
 cudaError_t launch_lateral_c2c(const float2* in, float2* out, int L, int C, int outer, bool inverse, const float2* tw,
-                               int twstride, cudaStream_t s, int n) {
-  if (inverse) return lat_any<kLatC2CInv>(in, out, L, C, outer, tw, twstride, s, n);
-  return lat_any<kLatC2C>(in, out, L, C, outer, tw, twstride, s, n);
+                               int twstride, cudaStream_t s, bool pdl, int n) {
+  if (inverse) return lat_any<kLatC2CInv>(in, out, L, C, outer, tw, twstride, s, pdl, n);
+  return lat_any<kLatC2C>(in, out, L, C, outer, tw, twstride, s, pdl, n);
 }
 
 // In-place FFT of contiguous lines (the depth transform of Eq. fft-1 and its
@@ -259,6 +259,7 @@ __global__ void __launch_bounds__(1024) rows_fft_kernel(float2* data, int L, int
   const bool valid = row < rows;
   float2* X = smem + slot * rows_slot(L);
   float2* line = data + (size_t)(valid ? row : 0) * L;
+  pdl_wait();
   {
     constexpr int R = 16;
     const int LR = L / R;
@@ -279,7 +280,7 @@ __global__ void __launch_bounds__(1024) rows_fft_kernel(float2* data, int L, int
 }
 
 cudaError_t launch_rows_c2c(float2* data, int L, int rows, bool inverse, const float2* tw, int twstride,
-                            cudaStream_t s) {
+                            cudaStream_t s, bool pdl) {
   if (L < 32 || (L & (L - 1)) != 0 || L / kElemsPerThread > 1024) return cudaErrorInvalidValue;
   int mshift = 0;
   while ((1 << mshift) < L) ++mshift;
@@ -288,17 +289,10 @@ cudaError_t launch_rows_c2c(float2* data, int L, int rows, bool inverse, const f
   const int rpc = threads / tpr;
   const size_t smem = (size_t)rpc * rows_slot(L) * sizeof(float2);
   const int ctas = (rows + rpc - 1) / rpc;
-  cudaError_t e;
-  if (inverse) {
-    e = cudaFuncSetAttribute(rows_fft_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    rows_fft_kernel<true><<<ctas, threads, smem, s>>>(data, L, mshift, rows, tw, twstride);
-  } else {
-    e = cudaFuncSetAttribute(rows_fft_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    rows_fft_kernel<false><<<ctas, threads, smem, s>>>(data, L, mshift, rows, tw, twstride);
-  }
-  return cudaGetLastError();
+  void (*k)(float2*, int, int, int, const float2*, int) = inverse ? rows_fft_kernel<true> : rows_fft_kernel<false>;
+  const cudaError_t e = allow_smem(k, smem);
+  if (e != cudaSuccess) return e;
+  return launch_kernel(k, dim3(ctas), dim3(threads), smem, s, pdl, data, L, mshift, rows, tw, twstride);
 }
 
 // The depth stage of the forward model: lines of n image layers, zero-padded to
@@ -317,6 +311,7 @@ __global__ void __launch_bounds__(1024) rows_fold_kernel(const float2* __restric
   const bool valid = row < rows;
   float2* X = smem + slot * rows_slot(L);
   const float2* line = in + (size_t)(valid ? row : 0) * n;
+  pdl_wait();
   float2 v[kElemsPerThread];
   if (2 * n <= L && mshift >= 9 && ((mshift - 5) & 3) == 0) {
     // L = 32 16^k: a radix-32 first pass leaves radix-16 passes only (no radix-2
@@ -356,7 +351,7 @@ __global__ void __launch_bounds__(1024) rows_fold_kernel(const float2* __restric
 }
 
 cudaError_t launch_rows_fold(const float2* in, int n, float2* out, int L, int rows, const float2* tw, int twstride,
-                             cudaStream_t s) {
+                             cudaStream_t s, bool pdl) {
   if (L < 32 || (L & (L - 1)) != 0 || L / kElemsPerThread > 1024) return cudaErrorInvalidValue;
   int mshift = 0;
   while ((1 << mshift) < L) ++mshift;
@@ -364,10 +359,10 @@ cudaError_t launch_rows_fold(const float2* in, int n, float2* out, int L, int ro
   const int threads = tpr > 128 ? tpr : 128;
   const int rpc = threads / tpr;
   const size_t smem = (size_t)rpc * rows_slot(L) * sizeof(float2);
-  const cudaError_t e = cudaFuncSetAttribute(rows_fold_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(rows_fold_kernel, smem);
   if (e != cudaSuccess) return e;
-  rows_fold_kernel<<<(rows + rpc - 1) / rpc, threads, smem, s>>>(in, n, out, L, mshift, rows, tw, twstride);
-  return cudaGetLastError();
+  return launch_kernel(rows_fold_kernel, dim3((rows + rpc - 1) / rpc), dim3(threads), smem, s, pdl, in, n, out, L,
+                       mshift, rows, tw, twstride);
 }
 
 }  // namespace pai

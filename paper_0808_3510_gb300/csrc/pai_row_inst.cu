@@ -16,16 +16,15 @@ namespace pai {
 template <typename K>
 static cudaError_t launch_k(K kernel, const RowLaunch& L, const WindowPoly& w, int threads, int ctas, size_t smem,
                            cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kernel, smem);
   if (e != cudaSuccess) return e;
-  kernel<<<ctas, threads, smem, s>>>(L, w);
-  return cudaGetLastError();
+  return launch_kernel(kernel, dim3(ctas), dim3(threads), smem, s, L.pdl, L, w);
 }
 
 template <typename K>
 static int occ_k(K kernel, int threads, size_t smem) {
   int n = 0;
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+  if (allow_smem(kernel, smem) != cudaSuccess) return 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) != cudaSuccess) return 0;
   return n;
 }

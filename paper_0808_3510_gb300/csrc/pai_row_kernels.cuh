@@ -1105,6 +1105,7 @@ template <int H, bool ZF, bool PAIRED = false>
 __global__ void __launch_bounds__(1024) row_forward_kernel(RowLaunch L, WindowPoly W) {
   extern __shared__ float2 smem[];
   __shared__ int s_item;
+  pdl_wait();
   for (int item = blockIdx.x; item < L.nitems; item = next_item(L, &s_item)) {
     const WorkItem wi = L.items[item];
     const RowProblem& P = L.problems[wi.problem];
@@ -1602,6 +1603,7 @@ template <int H, bool ZF>
 __global__ void __launch_bounds__(1024) row_adjoint_pairs_kernel(RowLaunch L, WindowPoly W) {
   extern __shared__ float2 smem[];
   __shared__ int s_item;
+  pdl_wait();
   for (int item = blockIdx.x; item < L.nitems; item = next_item(L, &s_item)) {
     const WorkItem wi = L.items[item];
     const RowProblem& P = L.problems[wi.problem];
@@ -1647,6 +1649,7 @@ template <int H, bool PAIR>
 __global__ void __launch_bounds__(1024) row_model_kernel(RowLaunch L, WindowPoly W) {
   extern __shared__ float2 smem[];
   __shared__ int s_item;
+  pdl_wait();
   constexpr int kShift = kCellShift<PAIR>;
   for (int item = blockIdx.x; item < L.nitems; item = next_item(L, &s_item)) {
     const WorkItem wi = L.items[item];
@@ -1779,6 +1782,7 @@ template <int H, bool ZF>
 __global__ void __launch_bounds__(1024) row_adjoint_kernel(RowLaunch L, WindowPoly W) {
   extern __shared__ float2 smem[];
   __shared__ int s_item;
+  pdl_wait();
   float4* nodes_all = reinterpret_cast<float4*>(smem + L.fft_region);
   for (int item = blockIdx.x; item < L.nitems; item = next_item(L, &s_item)) {
     const WorkItem wi = L.items[item];

@@ -51,3 +51,25 @@ def test_window_left_open_on_a_tiny_problem(pai):
     g = ph.Geometry(dim=2, nx=4, nt=8, nz=6)
     h = ph.random_image(23, g).astype(np.float32)
     assert rel(to_np(pai.Plan(gdict(g)).adjoint(to_gpu(h))), oracle.adjoint(g, h.astype(np.float64))) < TOL
+
+
+@pytest.mark.parametrize("kw", [dict(dim=2, nx=54, nt=66, nz=30), dict(dim=2, nx=64, nt=128, nz=64)], ids=["cufft", "own"])
+def test_calls_from_fresh_threads_and_new_buffers(pai, kw):
+    """A plan's first calls launch directly and repeated ones replay a graph: the same bits either way, on changing
+    buffers and from a thread that has made no CUDA call before."""
+    import threading
+
+    import torch
+    g = ph.Geometry(**kw)
+    plan = pai.Plan(gdict(g, K=3))
+    ps = [to_gpu(ph.random_data(30 + i, g)) for i in range(3)]
+    outs = [torch.empty(g.image_shape, device="cuda") for _ in range(2)]
+    ref = [plan.reconstruct(p).clone() for p in ps]
+    for i in range(24):  # every pair of buffers four times
+        assert torch.equal(plan.reconstruct(ps[i % 3], out=outs[i % 2]), ref[i % 3])
+    h = to_gpu(ph.random_image(40, g))
+    got = []
+    t = threading.Thread(target=lambda: got.append(plan.adjoint(h).clone()))
+    t.start()
+    t.join()
+    assert len(got) == 1 and torch.equal(got[0], plan.adjoint(h))
