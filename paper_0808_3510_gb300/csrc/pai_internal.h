@@ -98,7 +98,7 @@ struct RowProblem {
   int tpr;                 // threads per row in the FFT = M / kElemsPerThread
   int rpc;                 // rows per CTA work item
   int slot;                // complex values per row slot in shared memory (row_slot_stride(M)): band spreads
-  int slot32;           // the same with one pad per 32: forward kernel and the adjoint's list spreads
+  int slot32;              // the same with one pad per 32: forward kernel and the adjoint's list spreads
   float B2hi, B2lo;        // (M c dt)^2 as float-float: node x = B sqrt(S + az)
   float wscale;            // 2 c dt/dz * B / (n1 n2 nz): W = wscale * kz / x
   float nt_over_M;         // for the node phase

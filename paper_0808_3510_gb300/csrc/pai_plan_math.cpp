@@ -148,13 +148,13 @@ void fill_row_tables(const pai_geometry& g, double c_eff, int H, double beta, fl
 }
 
 void band_layout(double cells, int H, int shift, int warps, long long fft, int& ps, int& slot) {
-  // 2H window cells and a few to spare; the phases start 2 (mod 8) 16-byte or 4 (mod 16) 8-byte cells apart, so that
+  // 2H window cells, two a pass over two nodes may touch beyond, and a few to spare; the phases start 2 (mod 8) 16-byte or 4 (mod 16) 8-byte cells apart, so that
   // neighbouring nodes one, two or four cells apart fall on distinct banks
-  const int n = (int)std::min(1e7, std::ceil(cells)) + 2 * H + 8;
+  const int n = (int)std::min(1e7, std::ceil(cells)) + 2 * H + 10;
   const int period = 128 >> shift, off = period / 4;
   ps = (n + 3) / 4;
   ps += ((off - ps % period) + period) % period;
-  const long long bytes = ((4LL * ps + (warps > 1 ? warps * (2 * H + 4) : 0)) << shift) + 8LL * warps;
+  const long long bytes = ((4LL * ps + (warps > 1 ? warps * (2 * H + 6) : 0)) << shift) + 8LL * warps;
   const long long need = std::max(fft, (bytes + 7) / 8);
   slot = (int)std::min<long long>(1 << 28, (need + 1) & ~1LL);
 }

@@ -180,6 +180,28 @@ __device__ __forceinline__ void dft_reg(float2 (&v)[R]) {
   for (int i = 0; i < R; ++i) v[i] = a[i];
 }
 
+// Shared-memory accesses by 32-bit address.
+__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ float4 lds4(unsigned a) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(a)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 lds2(unsigned a) {
+  float2 v;
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void sts2(unsigned a, float2 v) {
+  asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void sts4(unsigned a, float4 v) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+
 // Layouts of a row slot in shared memory.  Passes between the first and the
 // last keep one padding element every 16 or 32 (padi) so strided butterfly accesses
 // do not collide in the banks.  The last pass of the forward transform writes
@@ -540,28 +562,6 @@ __device__ __forceinline__ void fft_rest(float2* X, int M, int mshift, int lane,
   if (rem == 3) fft_pass<8, INV, OUT, CHAIN_R, PS>(X, M, Ns, lane, tpr, tw, twstride, active);
   else if (rem == 2) fft_pass<4, INV, OUT, CHAIN_R, PS>(X, M, Ns, lane, tpr, tw, twstride, active);
   else if (rem == 1) fft_pass<2, INV, OUT, CHAIN_R, PS>(X, M, Ns, lane, tpr, tw, twstride, active);
-}
-
-// 16-byte shared-memory accesses by 32-bit address (the band grid below).
-__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ float4 lds4(unsigned a) {
-  float4 v;
-  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "r"(a)
-               : "memory");
-  return v;
-}
-__device__ __forceinline__ float2 lds2(unsigned a) {
-  float2 v;
-  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
-  return v;
-}
-__device__ __forceinline__ void sts2(unsigned a, float2 v) {
-  asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
-}
-__device__ __forceinline__ void sts4(unsigned a, float4 v) {
-  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
 
 // The band grid of an adjoint row (written by the pair spread, see
@@ -1451,7 +1451,9 @@ __device__ __forceinline__ void band_spread2(const WindowPoly& W, const BandTaps
 // others the warp owns alone, so it zeroes them and begins without a barrier.
 template <int H>
 struct BandPart {
-  static constexpr int kSpill = 2 * H + 4;
+  // a pass over two nodes adds (zeros) up to kReach cells beyond the second one's last
+  static constexpr int kReach = 2;
+  static constexpr int kSpill = 2 * H + 4 + kReach;  // at most 32
   int nw, wa, w;       // warps, warps with nodes, this warp
   int gw, l;           // lanes per row in a warp, this lane's place
   int n0, n1;          // this warp's nodes
@@ -1490,9 +1492,9 @@ __device__ __forceinline__ void band_begin(BandPart<H>& b, Band& band, char* slo
   const int j_first = b.nw > 1 ? __shfl_sync(full, j, 2) : j_row, j_prev = b.nw > 1 ? __shfl_sync(full, j, 3) : j_row;
   band.lo = j_row - H;
   b.lo_w = j_first - H;
-  b.hi_prev = b.w > 0 ? j_prev + H + 1 : -(1 << 30);
+  b.hi_prev = b.w > 0 ? j_prev + H + 1 + BandPart<H>::kReach : -(1 << 30);
   if (on) {
-    const int hi = j_last + H + 1;
+    const int hi = j_last + H + 1 + BandPart<H>::kReach;
     if (b.l == 0) b.bnd[b.w] = make_int2(b.lo_w, hi);
     const Cell<WIDE> zero = cell_zero<WIDE>();
     for (int c = (b.w > 0 ? b.hi_prev + 1 - band.lo : 0) + b.l; c <= hi - band.lo; c += b.gw)

@@ -73,3 +73,15 @@ def test_calls_from_fresh_threads_and_new_buffers(pai, kw):
     t.start()
     t.join()
     assert len(got) == 1 and torch.equal(got[0], plan.adjoint(h))
+
+
+@pytest.mark.parametrize("kw", [dict(dim=2, nx=60, nt=2000, nz=200, dt=0.9), dict(dim=3, nx=12, ny=10, nt=500, nz=40, dt=0.2)],
+                         ids=["2d", "3d"])
+def test_forward_model_repeats_bit_for_bit(pai, kw):
+    """Every cell belongs to one warp, also those a pass over two nodes touches beyond the last of them."""
+    import torch
+    g = ph.Geometry(**kw)
+    model = pai.ForwardModel(gdict(g, K=3))
+    f = to_gpu(ph.random_image(41, g))
+    ref = model(f).clone()
+    assert all(torch.equal(model(f), ref) for _ in range(20))
