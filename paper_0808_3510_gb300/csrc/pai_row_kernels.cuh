@@ -1624,6 +1624,48 @@ __global__ void __launch_bounds__(1024) row_adjoint_pairs_kernel(RowLaunch L, Wi
   }
 }
 
+// t a + conj(t) b
+__device__ __forceinline__ float2 model_sample(float2 t, float2 a, float2 b) {
+  return fma2(make_float2(t.x, t.x), cadd(a, b), mul2(make_float2(t.y, t.y), make_float2(b.y - a.y, a.x - b.x)));
+}
+
+// Last pass of the forward model's transform (radix R < 16, Ns = M/R) with its
+// samples g_n = t_n V[n] + conj(t_n) V[M - n], n < nt, formed in registers: M - n
+// of butterfly j's outputs j + r Ns are those of butterfly Ns - j, so a thread
+// takes the butterflies q and Ns - q together (q = 0: 0 and Ns/2, each its own
+// mirror).  Saves a write and two reads of the row in shared memory.
+template <int R>
+__device__ __forceinline__ void model_last(const float2* X, int M, int nt, int lane, int tpr,
+                                           const float2* __restrict__ tw, int twstride,
+                                           const float2* __restrict__ tab, float2* dst) {
+  const int Ns = M / R;
+#pragma unroll
+  for (int i = 0; i < 8 / R; ++i) {
+    const int q = lane + i * tpr;
+    const int ja = q, jb = q == 0 ? Ns >> 1 : Ns - q;
+    float2 a[R], b[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      a[r] = X[padi(ja + r * Ns)];
+      b[r] = X[padi(jb + r * Ns)];
+    }
+    TwBase<R> t;
+    tw_load<R>(t, tw, ja * twstride);
+    tw_apply<R, false>(a, t);
+    tw_load<R>(t, tw, jb * twstride);
+    tw_apply<R, false>(b, t);
+    dft_reg<R, false>(a);
+    dft_reg<R, false>(b);
+    if (!dst) continue;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int na = ja + r * Ns, nb = jb + r * Ns;
+      if (na < nt) dst[na] = model_sample(__ldg(&tab[na]), a[r], q == 0 ? a[(R - r) % R] : b[R - 1 - r]);
+      if (nb < nt) dst[nb] = model_sample(__ldg(&tab[nb]), b[r], q == 0 ? b[R - 1 - r] : a[R - 1 - r]);
+    }
+  }
+}
+
 // Forward-model row kernel (the operator Q of Sec. 2 on a padded periodic
 // box).  A row's samples are g_n = sum_j c_j cos(2 pi nu_j n / nt), j =
 // 0..nz/2, nu_j >= 0 the frequency of |K| (j = 0 included: its frequency is
@@ -1762,17 +1804,19 @@ __global__ void __launch_bounds__(1024) row_model_kernel(RowLaunch L, WindowPoly
       first_pass_regs<false>(X, v, lane);
     }
     __syncthreads();
-    fft_rest<false, kLayoutFlat>(X, M, P.mshift, lane, tpr, L.tw, L.Mmax >> P.mshift);
     const int row = sub ? row_b : (valid ? unit : -1);
-    if (row >= 0) {
-      float2* dst = const_cast<float2*>(P.pt) + (size_t)row * P.nt;
-      for (int n = lane; n < P.nt; n += tpr) {
-        const float2 t = __ldg(&P.model_tab[n]);
-        const float2 a = X[n], b = X[(M - n) & (M - 1)];
-        // t a + conj(t) b
-        dst[n] = fma2(make_float2(t.x, t.x), cadd(a, b),
-                      mul2(make_float2(t.y, t.y), make_float2(b.y - a.y, a.x - b.x)));
-      }
+    float2* dst = row >= 0 ? const_cast<float2*>(P.pt) + (size_t)row * P.nt : nullptr;
+    const int last = P.mshift & 3, tws = L.Mmax >> P.mshift;
+    if (last == 0) {
+      fft_rest<false, kLayoutFlat>(X, M, P.mshift, lane, tpr, L.tw, tws);
+      if (dst)
+        for (int n = lane; n < P.nt; n += tpr) dst[n] = model_sample(__ldg(&P.model_tab[n]), X[n], X[(M - n) & (M - 1)]);
+    } else {
+      for (int Ns = 16; Ns * 16 <= M; Ns <<= 4)
+        fft_pass<16, false, kLayoutPadded>(X, M, Ns, lane, tpr, L.tw, tws);
+      if (last == 1) model_last<2>(X, M, P.nt, lane, tpr, L.tw, tws, P.model_tab, dst);
+      else if (last == 2) model_last<4>(X, M, P.nt, lane, tpr, L.tw, tws, P.model_tab, dst);
+      else model_last<8>(X, M, P.nt, lane, tpr, L.tw, tws, P.model_tab, dst);
     }
   }
 }
