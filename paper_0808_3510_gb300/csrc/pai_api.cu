@@ -1,15 +1,16 @@
 // pai_api.cu -- plans and entry points of libpai (C ABI declared in include/pai.h).
 //
 // A call of pai_reconstruct runs Algorithm 2 as three stream-ordered stages:
-//   (a) cuFFT real-to-complex lateral transform of every problem (Eq. fft-1a),
-//       layout [row][n] with the halved lateral axis last;
+//   (a) lateral real-to-complex transform of every problem (Eq. fft-1a), by the
+//       library's kernels or cuFFT, layout [row][n] with the halved lateral
+//       axis last;
 //   (b) ONE persistent launch of the fused row kernel over every lateral
 //       frequency row of every problem (prescale, oversampled FFT, window
-//       gather, weight: Algorithm 1 + Eq. fft-0), writing the half image
-//       spectrum;
-//   (c) cuFFT complex-to-real inverse transform of every problem (Eq. fft-1).
-// The sequence is captured once per (input, output) pointer pair into a CUDA
-// graph and replayed.  pai_adjoint runs the transposed stages in reverse.
+//       gather, weight: Algorithm 1 + Eq. fft-0), writing the image spectrum;
+//   (c) inverse transform of every problem (Eq. fft-1), likewise.
+// The stages are launched on the caller's stream or, where that is faster
+// (pai_plan_s::graphed), captured into a CUDA graph per (input, output) pointer
+// pair and replayed.  pai_adjoint runs the transposed stages in reverse.
 #include <cuda_runtime.h>
 #include <cufft.h>
 
@@ -89,15 +90,16 @@ struct pai_plan_s {
   bool pdl() const { return nbranch <= 1; }  // one stream: kernels launch as programmatic dependents
   // Whether repeated calls replay a graph.  A single problem on the library's
   // kernels is four to six launches: as programmatic dependents on the caller's
-  // stream they follow each other (and the previous call) closer than graph
-  // replays do (128^3: 53.8 us a pass against 60.7 with a graph; 2048x4096: 97.7
-  // and 104.2), unless the problem is so small that the launches themselves take
-  // longer than the kernels (128x256: 20.9 and 17.2 us; the two meet near 20 us a
-  // pass, about a million samples and voxels).  Calls of many cuFFT launches and
-  // of batches replay a graph.
+  // stream they follow the previous call closer than graph replays do (2048x4096:
+  // 97.7 us a pass against 104.2 with a graph, its adjoint 138 and 144), but they
+  // take the host 20 to 25 us instead of 10, and about 50 us more in a gradient
+  // step, whose adjoint runs on autograd's thread (128^3: 209 against 156 us a
+  // step, all of it host time).  So they are direct where the kernels of such a
+  // step outlast its host time of about 200 us: from some ten million samples and
+  // voxels.  Calls of many cuFFT launches and of batches replay a graph.
   bool graphed(bool adjoint) const {
     if (!use_graph) return false;
-    return probs.size() > 1 || !(adjoint ? zf_adj : zf) || data_total + img_total < ((size_t)1 << 20);
+    return probs.size() > 1 || !(adjoint ? zf_adj : zf) || data_total + img_total < ((size_t)10 << 20);
   }
   WindowPoly poly{};
   double beta = 0, pred_err = 0, fit_err = 0;
@@ -538,6 +540,20 @@ pai_status enqueue_adjoint(pai_plan_s* P, const float* d_h, float* d_pbar, cudaS
   return enqueue_last(P, d_pbar, s, true);
 }
 
+// A plan's calls are not part of a caller's stream capture (PAI_USE_GRAPH=0
+// plans excepted): a graph of the caller's would hold the plan's workspace beyond
+// pai_destroy.  Refused before anything is launched, so that the capture stays
+// whole, and alike for calls that launch directly and calls that replay a graph.
+bool in_callers_capture(pai_plan_s* P) {
+  if (!P->use_graph) return false;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(P->stream, &cs) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return cs != cudaStreamCaptureStatusNone;
+}
+
 pai_status run(pai_plan_s* P, const void* in, void* out, bool adjoint) {
   int prev = 0;
   cudaGetDevice(&prev);
@@ -545,10 +561,10 @@ pai_status run(pai_plan_s* P, const void* in, void* out, bool adjoint) {
   // CUDA call yet (autograd's backward threads) this makes its context current,
   // which a direct cuFFT execution needs
   cudaSetDevice(P->device);
-  pai_status st = PAI_OK;
+  pai_status st = in_callers_capture(P) ? PAI_ERR_CUDA : PAI_OK;
   GraphEntry* hit = nullptr;
   bool direct = !P->graphed(adjoint);
-  if (!direct) {
+  if (st == PAI_OK && !direct) {
     for (auto& ge : P->graphs)
       if (ge.in == in && ge.out == out && ge.adjoint == adjoint) hit = &ge;
     if (!hit) {
@@ -561,10 +577,10 @@ pai_status run(pai_plan_s* P, const void* in, void* out, bool adjoint) {
       if (direct) P->seen[P->seen_next++ % 8] = now;
     }
   }
-  if (direct) {
+  if (st == PAI_OK && direct) {
     st = adjoint ? enqueue_adjoint(P, (const float*)in, (float*)out, P->stream)
                  : enqueue_forward(P, (const float*)in, (float*)out, P->stream, false);
-  } else {
+  } else if (st == PAI_OK) {
     if (!hit) {
       // capture on the private stream (the caller's stream may be the legacy default stream)
       st = set_fft_streams(P, P->cap_stream);
@@ -1786,7 +1802,8 @@ pai_status pai_forward_model(pai_plan_t plan, const float* d_f, float* d_p) {
   const int ny = gi.dim == 3 ? gi.ny : 1;
   // plain launches, not a graph kept per pointer pair: four to six kernels of a
   // call that takes longer than their launches, and no capture on new buffers
-  pai_status st = enqueue_adjoint(plan, d_f, d_p, plan->stream);
+  pai_status st = in_callers_capture(plan) ? PAI_ERR_CUDA : PAI_OK;
+  if (st == PAI_OK) st = enqueue_adjoint(plan, d_f, d_p, plan->stream);
   if (st == PAI_OK) plan->own_kernels += plan->own_kernels_per_adj;
   if (st == PAI_OK && plan->d_cut) {
     // the data model g = w_cut * (Q f): only the samples near the faces are touched
