@@ -484,8 +484,8 @@ def fp32_fma_peak(dev, clocks):
 FORWARD_CONFIGS = {
     "forward3d": "3-D: 128^3 initial pressure (1-20 uniform balls) -> 128 x 128 detectors x 256 samples",
     "forward2d": "2-D: 2048 x 2048 initial pressure (50 f_circ discs) -> 2048 detectors x 4096 samples",
-    "datamodel2d": "2-D partial data g = w_cut Q f (Eq. data-part): forward2d with the cutoff eps = 16 fused into "
-                   "the copy of the detector rows",
+    "datamodel2d": "2-D partial data g = w_cut Q f (Eq. data-part): forward2d with the cutoff eps = 16 "
+                   "applied in place",
 }
 
 
@@ -560,7 +560,7 @@ def run_forward_model(args, rank, world, local_rank):
     st = model.profile_stages(reps=20)
     bx, by, bz = model.box
     rows = bx * (by // 2 + 1) if g.dim == 3 else bx // 2 + 1
-    nbytes_alg = rows * (bz + g.nt) * 8  # depth spectrum rows in, temporal rows out
+    nbytes_alg = rows * (bz // 2 + 1 + g.nt) * 8  # folded depth spectrum rows in, temporal rows out
     peak, peak_src = hbm_peak()
     achieved = nbytes_alg / (st[1] * 1e-3) / 1e9
     if rank == 0:
@@ -574,8 +574,8 @@ def run_forward_model(args, rank, world, local_rank):
             "step": "forward model (image -> detector data)",
             "parity": {"checked_by": "tests/test_gpu_cutoff.py::test_data_model_against_oracle"
                        if args.config == "datamodel2d" else "tests/test_gpu_forward.py", "bar_rel_l2": 1e-5},
-            "roofline": {"bound": "hbm", "kernel": "row_adjoint in forward-model mode (node pairs, spread, inverse "
-                         "FFT, crop)", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
+            "roofline": {"bound": "hbm", "kernel": "row_model (node pairs into band grids, cosine transform, "
+                         "crop)", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                          "traffic": None, "peak_source": peak_src, "algorithmic_bytes_per_launch": nbytes_alg,
                          "kernel_ms": st[1], "stage_ms": {"image_fft": st[0], "row_kernel": st[1],
                                                            "lateral_inverse_fft": st[2]}},

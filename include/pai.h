@@ -51,7 +51,8 @@ typedef enum {
   PAI_ERR_INVALID_ARG = 1,  /* bad geometry, size or pointer                 */
   PAI_ERR_UNSUPPORTED = 2,  /* valid but outside what this build implements  */
   PAI_ERR_OOM = 3,          /* device or host allocation failed              */
-  PAI_ERR_CUDA = 4,         /* a CUDA runtime call or kernel launch failed   */
+  PAI_ERR_CUDA = 4,         /* a CUDA runtime call or kernel launch failed, or
+                               the plan's stream is being captured           */
   PAI_ERR_CUFFT = 5,        /* a cuFFT call failed                           */
   PAI_ERR_TIMEOUT = 6       /* a bounded device-side wait gave up            */
 } pai_status;
@@ -115,7 +116,8 @@ typedef struct {
   long long nodes;        /* nodes evaluated per call (sum over the batch)      */
   size_t workspace_bytes; /* device bytes owned by the plan                     */
   int uses_graph;         /* 1 if reconstructions or adjoints replay a captured
-                             CUDA graph (plans that run cuFFT, batches)         */
+                             CUDA graph (plans that run cuFFT, batches, all but
+                             large problems)                                   */
   int library_ffts;       /* bit 0: pai_reconstruct runs every stage on the
                              library's own kernels (power-of-two sizes, chosen
                              by the tuner), else its inverse uses cuFFT; bit 1:
@@ -137,7 +139,7 @@ pai_status pai_plan(const pai_geometry* g, void* cuda_stream, pai_plan_t* out);
 /* Create one plan for `count` independent 2-D or 3-D problems (g[0..count-1])
  * executed together: one lateral FFT per problem, ONE persistent row-kernel
  * launch over every lateral-frequency row of every problem, one inverse FFT
- * per problem, all replayed as one CUDA graph.  The problems share the tap
+ * per problem, replayed as one CUDA graph when called again on its buffers.  The problems share the tap
  * count and the method (PAI_ERR_INVALID_ARG otherwise); each keeps its own
  * oversampling.  When every problem leaves the window open (method KB, K,
  * oversampling and alpha all 0) the plan times window candidates -- for each
@@ -214,24 +216,24 @@ pai_status pai_profile_stages(pai_plan_t plan, const float* d_in, float* d_out, 
 pai_status pai_set_stream(pai_plan_t plan, void* cuda_stream);
 
 /* Spread of pai_adjoint and pai_forward_model (the transpose of the window
- * gather, Algorithm 1 read backwards).  Five spreads exist:
+ * gather, Algorithm 1 read backwards).  Spreads of pai_adjoint:
  *   atomic        shared-memory atomic adds per node (every node adds its 2H
  *                 tap contributions to the oversampled grid at once);
  *   runs          the same per run (the first node of each run of nodes on
  *                 the same grid cell sums the run and adds once per tap);
  *   tap           tap phases (nodes add tap by tap in a fixed order, one
  *                 barrier per phase);
- *   pairs         the nodes +-nu of a row as pairs, spread by one warp per row
- *                 (32 pairs at a time, runs summed by warp shuffles, plain
- *                 read-modify-writes; windowed methods, rows of 32 or 64
- *                 threads);
- *   pairs_atomic  the same by every warp of the row, adding with shared-memory
- *                 atomics (windowed methods).
- * tap and pairs are bit-identical on repeated calls; for the three atomic
+ *   pairs         the nodes +-nu of a row as pairs that share one weight and
+ *                 one cell of a grid covering only the cells the row reaches;
+ *                 every warp owns its cells, so plain read-modify-writes in a
+ *                 fixed order (windowed methods).
+ * tap and pairs are bit-identical on repeated calls; for the two atomic
  * spreads the order of the additions into one grid cell, hence the last bits
  * of the result, may differ from call to call.  pai_plan times every spread
  * that applies and keeps the fastest (the environment variable PAI_SPREAD
- * forces one by the names above).
+ * forces one by the names above; "pairs_atomic", an earlier variant, selects
+ * pairs).  pai_forward_model runs a row kernel of its own, bit-identical on
+ * repeated calls, unless one of the first three is forced.
  * deterministic = 1: the faster of tap and pairs; deterministic = 0: back to
  * the plan's choice.  pai_reconstruct is deterministic either way.  Waits for
  * the plan's stream and drops the plan's captured CUDA graphs (they are

@@ -25,7 +25,8 @@ namespace pai {
 // half-warp in the load and store phases, FP columns times 16 / FP consecutive
 // elements, then fall on 16 different banks, in the first pass's writes too
 // (17 x0 + r).  (One pad per 32 and a shift of 4 made those accesses two- to
-// four-way conflicts.)
+// four-way conflicts: the eight lateral passes of a 256^3 gradient took 356 us
+// against 316 now, of 240 their bytes need at the measured copy rate.)
 __host__ __device__ constexpr int lateral_slot(int L, int FP) {
   const int s = L + (L >> 4);
   return s + (16 / FP - s % 16 + 16) % 16;
@@ -46,7 +47,9 @@ __device__ __forceinline__ float2 ldg_pair(const float2* p, int pairs) {
 // PRUNED: only the first n of the L points exist on the real side (R2C, C2R)
 // or on the input of the C2C / the output of the inverse C2C; the others are
 // zeros, or are not stored.  The forward model's box is two to four times the
-// image per axis, so most of its traffic is such points.  (Compiled apart: the
+// image per axis, so most of its traffic is such points: the lateral passes of a
+// 128^3 volume in its 512^3 box took 852 us on the whole box, 203 us pruned (and
+// with them went 345 us of padding and 18 us of cropping).  (Compiled apart: the
 // full kernel keeps its loads without the extra predicate.)  pairs = 0: the
 // real buffer is only 4-byte aligned (the forward model takes such buffers;
 // the plans' other calls ask for 8 bytes), its floats move one at a time.

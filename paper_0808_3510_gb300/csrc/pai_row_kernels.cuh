@@ -19,7 +19,7 @@
 // The oversampled spectrum of a row therefore never reaches HBM: a row costs
 // one read of its nt complex samples and one write of its nz/2+1 (or twice
 // that) spectrum values.  The adjoint kernel runs the exact transpose of the
-// same steps in reverse order (spread in gather form, inverse FFT, prescale).
+// same steps in reverse order (spread, inverse FFT, prescale).
 //
 // Conventions fixed by the design (each traced to the paper):
 //  * the constant of Fourmont's identity is 1/(2 pi c) (it is the Fourier
@@ -1553,9 +1553,15 @@ __device__ __forceinline__ void band_end(const BandPart<H>& b, Band& band, int l
 // pair's values are formed right before they are spread (no list in shared
 // memory).
 //
-// What bounds it: shared-memory accesses, 32 bytes per tap and pair.  The
-// lists and float atomics it replaces held one CTA per SM for long rows and
-// serialised on equal cells.
+// What bounds it: instruction issue (57 % of the slots) and shared-memory
+// accesses (69 % of their peak; 32 bytes per tap and pair) about equally, behind
+// them the latency of the tap chain; 64 registers at 32 warps per SM measured
+// best (56: +6 %, 90 and half the warps: +16 %).  The lists, run sums and float
+// atomics it replaced held one CTA per SM for long rows and serialised on equal
+// cells: 2048x4096 (M = 8192, H = 8) 126 -> 91 us, 256^3 (M = 1024, H = 6) 224 ->
+// 221 us, 666x1500 (M = 4096) 21.6 -> 18.3 us.  Spreading two pairs per lane as
+// the forward model does paid at 256^3 (216 us) but not for longer rows or wider
+// windows (105 and 19.6 us), whose weights leave the registers.
 template <int H, bool ZF>
 __device__ __forceinline__ bool adjoint_band(const RowProblem& P, const WindowPoly& W, int row, bool valid, int lane,
                                              float2* X, Band& band) {
@@ -1687,8 +1693,13 @@ __device__ __forceinline__ void model_last(const float2* X, int M, int nt, int l
 // of 2 tpr threads spreads both rows' values with one set of weights into
 // 16-byte cells, then transforms one row with each half of its threads.
 //
-// What bounds it: instruction issue (about a third of it node positions and
-// weights) and shared-memory accesses.
+// What bounds it: shared-memory accesses (79 % of their peak) and instruction
+// issue (64 % of the slots), about a third of it node positions and weights.
+// 128^3 in its 512^3 box (131 584 rows, M = 512): 1264 us with the node pairs of
+// the adjoint and their lists, 957 us with them in band grids, 675 us as this
+// kernel, 604 us with two nodes per lane (band_spread2); 2048x4096 in 8192^2
+// (4097 rows, M = 8192): 1455, 584, 602 and 477 us; with the last pass forming
+// the samples (model_last) another 27 us less each.
 template <int H, bool PAIR>
 __global__ void __launch_bounds__(1024) row_model_kernel(RowLaunch L, WindowPoly W) {
   extern __shared__ float2 smem[];
