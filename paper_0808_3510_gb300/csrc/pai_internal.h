@@ -38,7 +38,11 @@ inline cudaError_t allow_smem(K* kernel, size_t smem) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 #ifdef __CUDACC__
-// First statement of a kernel: waits for the previous one.  (The next kernel's
+// First statement of a kernel: waits for the previous one.  What an earlier
+// kernel or the caller wrote is then loaded plainly, never by __ldg or through a
+// const __restrict__ parameter: those promise data that nobody writes while this
+// kernel runs, which begins before the previous one ends, and the compiler may
+// move them above the wait.  (Tables uploaded with the plan may.)  (The next kernel's
 // CTAs come when this one's leave; letting them in earlier,
 // griddepcontrol.launch_dependents, had them hold shared memory while they
 // waited: 128^3 65.7 against 60.7 us, 128x256 18.7 against 17.2 us.)

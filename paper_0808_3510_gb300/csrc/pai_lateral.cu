@@ -38,10 +38,10 @@ enum : int { kLatR2C = 0, kLatC2R = 1, kLatC2C = 2, kLatC2CInv = 3 };
 
 // Two adjacent floats, one load when they start on an 8-byte boundary (pairs).
 template <bool CHECK>
-__device__ __forceinline__ float2 ldg_pair(const float2* p, int pairs) {
-  if (!CHECK || pairs) return __ldg(p);
+__device__ __forceinline__ float2 load_pair(const float2* p, int pairs) {
+  if (!CHECK || pairs) return *p;
   const float* q = reinterpret_cast<const float*>(p);
-  return make_float2(__ldg(q), __ldg(q + 1));
+  return make_float2(q[0], q[1]);
 }
 
 // PRUNED: only the first n of the L points exist on the real side (R2C, C2R)
@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(1024) lateral_kernel(const void* vin, void* vo
     float2 z[kElemsPerThread];
 #pragma unroll
     for (int i = 0; i < kElemsPerThread; ++i)
-      z[i] = live && (!PRUNED || x0 + i * xs < n) ? ldg_pair<PRUNED>(src + (size_t)i * xs * (C / 2), pairs)
+      z[i] = live && (!PRUNED || x0 + i * xs < n) ? load_pair<PRUNED>(src + (size_t)i * xs * (C / 2), pairs)
                                                   : make_float2(0.f, 0.f);
     first_pass_regs<false>(Z, z, x0);
   } else if (KIND == kLatC2C || KIND == kLatC2CInv) {
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(1024) lateral_kernel(const void* vin, void* vo
 #pragma unroll
     for (int i = 0; i < NK; ++i) {
       const int k = x0 + i * xs;
-      abv[i] = (live && k <= half) ? __ldg(reinterpret_cast<const float4*>(in + (size_t)k * C + c0 + 2 * f))
+      abv[i] = (live && k <= half) ? *reinterpret_cast<const float4*>(in + (size_t)k * C + c0 + 2 * f)
                                    : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 #pragma unroll
@@ -303,9 +303,8 @@ cudaError_t launch_rows_c2c(float2* data, int L, int rows, bool inverse, const f
 // node pair carries the sum), so a line costs n values read and L/2 + 1
 // written instead of L read and L written, and the padded box itself is never
 // in memory.
-__global__ void __launch_bounds__(1024) rows_fold_kernel(const float2* __restrict__ in, int n, float2* __restrict__ out,
-                                                         int L, int mshift, int rows, const float2* __restrict__ tw,
-                                                         int twstride) {
+__global__ void __launch_bounds__(1024) rows_fold_kernel(const float2* in, int n, float2* out, int L, int mshift,
+                                                         int rows, const float2* __restrict__ tw, int twstride) {
   extern __shared__ float2 smem[];
   const int tpr = L / kElemsPerThread;
   const int slot = threadIdx.x / tpr;
@@ -325,7 +324,7 @@ __global__ void __launch_bounds__(1024) rows_fold_kernel(const float2* __restric
 #pragma unroll
     for (int r = 0; r < kElemsPerThread; ++r) {
       const int z = j + r * L32;
-      v[r] = z < n ? __ldg(line + z) : make_float2(0.f, 0.f);
+      v[r] = z < n ? line[z] : make_float2(0.f, 0.f);
     }
     if (h) tw32_all(v);
     dft_reg<16, false>(v);
@@ -338,7 +337,7 @@ __global__ void __launch_bounds__(1024) rows_fold_kernel(const float2* __restric
 #pragma unroll
     for (int r = 0; r < kElemsPerThread; ++r) {
       const int z = lane + r * tpr;
-      v[r] = z < n ? __ldg(line + z) : make_float2(0.f, 0.f);
+      v[r] = z < n ? line[z] : make_float2(0.f, 0.f);
     }
     first_pass_regs<false>(X, v, lane);
     __syncthreads();

@@ -385,9 +385,9 @@ __device__ __forceinline__ void fft_pass(float2* X, int M, int Ns, int lane, int
 // z1 = Z[k][m], z2 = Z[nx - k][m] with m = n/2:
 // sample 2m = (z1 + conj z2) / 2, sample 2m+1 = (z1 - conj z2) / (2i).
 template <bool PAIRED>
-__device__ __forceinline__ float2 row_sample(const float2* __restrict__ src, const float2* __restrict__ src2, int n) {
-  if (!PAIRED) return __ldg(&src[n]);
-  const float2 z1 = __ldg(&src[n >> 1]), z2 = __ldg(&src2[n >> 1]);
+__device__ __forceinline__ float2 row_sample(const float2* src, const float2* src2, int n) {
+  if (!PAIRED) return src[n];
+  const float2 z1 = src[n >> 1], z2 = src2[n >> 1];
   return (n & 1) ? make_float2(0.5f * (z1.y + z2.y), 0.5f * (z2.x - z1.x))
                  : make_float2(0.5f * (z1.x + z2.x), 0.5f * (z1.y - z2.y));
 }
@@ -399,9 +399,9 @@ __device__ __forceinline__ float2 row_sample(const float2* __restrict__ src, con
 // Proposition's phase is absorbed).  Writes padded.
 template <bool PAIRED = false>
 __device__ __forceinline__ void fft_first_pass_from_global(float2* X, int M, int nt, int lane, int tpr,
-                                                           const float2* __restrict__ src,
+                                                           const float2* src,
                                                            const float* __restrict__ prescale,
-                                                           const float2* __restrict__ src2 = nullptr) {
+                                                           const float2* src2 = nullptr) {
   constexpr int R = 16;
   float2 v[R];
   const int MR = M / R, mask = M - 1, h = nt >> 1;
@@ -488,9 +488,9 @@ __device__ __forceinline__ void tw32_all(float2 (&v)[16]) {
 // load the butterfly's 16 samples.  Writes padded: padi<5>(32 j + q) = 33 j + q.
 template <bool PAIRED>
 __device__ __forceinline__ void fft_first_pass32_from_global(float2* X, int M, int nt, int lane, int tpr,
-                                                             const float2* __restrict__ src,
+                                                             const float2* src,
                                                              const float* __restrict__ prescale,
-                                                             const float2* __restrict__ src2) {
+                                                             const float2* src2) {
   const int half = tpr >> 1, q4 = M >> 2, M32 = M >> 5;
   const int h = lane >= half ? 1 : 0;
   const int j = lane - h * half;
@@ -1744,9 +1744,9 @@ __global__ void __launch_bounds__(1024) row_model_kernel(RowLaunch L, WindowPoly
       return j0;
     });
     auto value = [&](int i) {
-      const float2 ya = __ldg(za + i);
+      const float2 ya = za[i];
       if constexpr (PAIR) {
-        const float2 yb = row_b >= 0 ? __ldg(zb + i) : make_float2(0.f, 0.f);
+        const float2 yb = row_b >= 0 ? zb[i] : make_float2(0.f, 0.f);
         return Cell<true>{make_float4(P.wscale * ya.x, P.wscale * ya.y, P.wscale * yb.x, P.wscale * yb.y)};
       } else {
         return Cell<false>{make_float2(P.wscale * ya.x, P.wscale * ya.y)};

@@ -1,0 +1,36 @@
+"""Rules the CUDA sources keep, read from the sources themselves (what they guard against shows on a GPU only now and
+then, or not with today's compiler)."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_0808_3510_gb300", "csrc")
+SOURCES = sorted(f for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh")))
+
+
+def _code(name):
+    with open(os.path.join(CSRC, name)) as f:
+        s = f.read()
+    return re.sub(r"//[^\n]*", "", re.sub(r"/\*.*?\*/", "", s, flags=re.S))
+
+
+def _kernels(code):
+    """(name, parameter list) of every __global__ function."""
+    for m in re.finditer(r"__global__\s+void\s+(?:__launch_bounds__\(\d+\)\s*)?(\w+)\(([^)]*)\)", code):
+        yield m.group(1), m.group(2)
+
+
+@pytest.mark.parametrize("name", SOURCES)
+def test_read_only_loads_are_of_plan_tables(name):
+    """A kernel launched as a programmatic dependent begins before the previous one ends: what that one may have
+    written must not be loaded as data that is constant while the kernel runs."""
+    code = _code(name)
+    tables = r"(tw|prescale|P\.zt|tab|P\.model_tab)\["
+    for m in re.finditer(r"__ldg\(([^;]*)", code):
+        arg = m.group(1)
+        assert re.match(r"&" + tables, arg) or re.match(r"T \+ ", arg), f"{name}: __ldg({arg[:40]}"
+    for kernel, params in _kernels(code):
+        for p in params.split(","):
+            if "__restrict__" in p and "const" in p:
+                assert p.split()[-1] == "tw", f"{name}: {kernel}: {p.strip()}"
