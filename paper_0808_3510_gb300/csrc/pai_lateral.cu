@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(1024) lateral_kernel(const void* vin, void* vo
                                                        int mshift, int C, long long in_outer, long long out_outer,
                                                        const float2* __restrict__ tw, int twstride, int n,
                                                        int pairs) {
-  extern __shared__ float2 smem[];
+  extern __shared__ __align__(16) float2 smem[];
   constexpr bool kInv = (KIND == kLatC2R || KIND == kLatC2CInv);
   const int tpr = L / kElemsPerThread;
   const int S = lateral_slot(L, FP);
@@ -253,7 +253,7 @@ cudaError_t launch_lateral_c2c(const float2* in, float2* out, int L, int C, int 
 template <bool INV>
 __global__ void __launch_bounds__(1024) rows_fft_kernel(float2* data, int L, int mshift, int rows,
                                                         const float2* __restrict__ tw, int twstride) {
-  extern __shared__ float2 smem[];
+  extern __shared__ __align__(16) float2 smem[];
   const int tpr = L / kElemsPerThread;
   const int slot = threadIdx.x / tpr;
   const int lane = threadIdx.x - slot * tpr;
@@ -305,7 +305,7 @@ cudaError_t launch_rows_c2c(float2* data, int L, int rows, bool inverse, const f
 // in memory.
 __global__ void __launch_bounds__(1024) rows_fold_kernel(const float2* in, int n, float2* out, int L, int mshift,
                                                          int rows, const float2* __restrict__ tw, int twstride) {
-  extern __shared__ float2 smem[];
+  extern __shared__ __align__(16) float2 smem[];
   const int tpr = L / kElemsPerThread;
   const int slot = threadIdx.x / tpr;
   const int lane = threadIdx.x - slot * tpr;

@@ -180,7 +180,8 @@ __device__ __forceinline__ void dft_reg(float2 (&v)[R]) {
   for (int i = 0; i < R; ++i) v[i] = a[i];
 }
 
-// Shared-memory accesses by 32-bit address.
+// Shared-memory accesses by 32-bit address (16 bytes at a time in the band grids: every kernel declares its
+// dynamic shared memory 16-byte aligned, which float2 alone does not make it).
 __device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ float4 lds4(unsigned a) {
   float4 v;
@@ -1103,7 +1104,7 @@ __device__ __forceinline__ int next_item(const RowLaunch& L, int* s_item) {
 // compiled apart so that the kernel of plans without them keeps its registers.
 template <int H, bool ZF, bool PAIRED = false>
 __global__ void __launch_bounds__(1024) row_forward_kernel(RowLaunch L, WindowPoly W) {
-  extern __shared__ float2 smem[];
+  extern __shared__ __align__(16) float2 smem[];
   __shared__ int s_item;
   pdl_wait();
   for (int item = blockIdx.x; item < L.nitems; item = next_item(L, &s_item)) {
@@ -1609,7 +1610,7 @@ __device__ __forceinline__ bool adjoint_band(const RowProblem& P, const WindowPo
 // own so that its register allocation does not carry the other schemes.
 template <int H, bool ZF>
 __global__ void __launch_bounds__(1024) row_adjoint_pairs_kernel(RowLaunch L, WindowPoly W) {
-  extern __shared__ float2 smem[];
+  extern __shared__ __align__(16) float2 smem[];
   __shared__ int s_item;
   pdl_wait();
   for (int item = blockIdx.x; item < L.nitems; item = next_item(L, &s_item)) {
@@ -1702,7 +1703,7 @@ __device__ __forceinline__ void model_last(const float2* X, int M, int nt, int l
 // the samples (model_last) another 27 us less each.
 template <int H, bool PAIR>
 __global__ void __launch_bounds__(1024) row_model_kernel(RowLaunch L, WindowPoly W) {
-  extern __shared__ float2 smem[];
+  extern __shared__ __align__(16) float2 smem[];
   __shared__ int s_item;
   pdl_wait();
   constexpr int kShift = kCellShift<PAIR>;
@@ -1837,7 +1838,7 @@ __global__ void __launch_bounds__(1024) row_model_kernel(RowLaunch L, WindowPoly
 // depth spectrum Fbar[row][l mod nz].
 template <int H, bool ZF>
 __global__ void __launch_bounds__(1024) row_adjoint_kernel(RowLaunch L, WindowPoly W) {
-  extern __shared__ float2 smem[];
+  extern __shared__ __align__(16) float2 smem[];
   __shared__ int s_item;
   pdl_wait();
   float4* nodes_all = reinterpret_cast<float4*>(smem + L.fft_region);

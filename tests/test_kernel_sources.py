@@ -34,3 +34,10 @@ def test_read_only_loads_are_of_plan_tables(name):
         for p in params.split(","):
             if "__restrict__" in p and "const" in p:
                 assert p.split()[-1] == "tw", f"{name}: {kernel}: {p.strip()}"
+
+
+@pytest.mark.parametrize("name", SOURCES)
+def test_dynamic_shared_memory_is_aligned_for_16_byte_cells(name):
+    """Row slots hold 16-byte cells and node records at offsets that are multiples of 16: the base has to be one."""
+    for m in re.finditer(r"extern\s+__shared__([^;]*);", _code(name)):
+        assert "__align__(16)" in m.group(1), f"{name}: extern __shared__{m.group(1)}"
