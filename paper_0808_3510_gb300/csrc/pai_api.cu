@@ -116,7 +116,7 @@ struct pai_plan_s {
   int nitems_fwd = 0;
   WorkItem* d_items_adj = nullptr;
   int nitems_adj = 0;
-  int* d_counter = nullptr;
+  unsigned* d_counter = nullptr;  // work counters: forward, adjoint by lists, by band grids, forward model
   void* d_cufft_work = nullptr;
   // batched plans: per-problem stages fork over branch streams (problem i on
   // branch i % nbranch), each branch with its own cuFFT work area
@@ -363,7 +363,7 @@ RowLaunch make_launch(pai_plan_s* P, bool adjoint) {
   L.problems = P->d_problems;
   L.items = adjoint ? P->d_items_adj : P->d_items_fwd;
   L.nitems = adjoint ? P->nitems_adj : P->nitems_fwd;
-  L.counter = P->d_counter + (adjoint ? 1 : 0);
+  L.counter = P->d_counter + (!adjoint ? 0 : P->spread_mode == 3 ? 2 : P->spread_mode == 4 ? 3 : 1);
   L.tw = P->d_tw;
   L.Mmax = P->TW;
   L.H = P->H;
@@ -920,8 +920,8 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
   PAI_TRY(plan_malloc(P, (void**)&P->d_tables, std::max<size_t>(tab_off, 4) * sizeof(float)));
   PAI_TRY(plan_malloc(P, (void**)&P->d_tw, tw.size() * sizeof(float2)));
   PAI_TRY(plan_malloc(P, (void**)&P->d_problems, count * sizeof(RowProblem)));
-  PAI_TRY(plan_malloc(P, (void**)&P->d_counter, 4 * sizeof(int)));
-  PAI_TRY(plan_zero(P, P->d_counter, 4 * sizeof(int)));
+  PAI_TRY(plan_malloc(P, (void**)&P->d_counter, 4 * sizeof(unsigned)));
+  PAI_TRY(plan_zero(P, P->d_counter, 4 * sizeof(unsigned)));
   PAI_TRY(plan_upload(P, P->d_tables, tables.data(), tab_off * sizeof(float)));
   PAI_TRY(plan_upload(P, P->d_tw, tw.data(), tw.size() * sizeof(float2)));
 

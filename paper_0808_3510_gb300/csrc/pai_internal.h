@@ -130,7 +130,7 @@ struct RowLaunch {
   const RowProblem* problems;  // device array
   const WorkItem* items;       // device array, ordered by decreasing cost
   int nitems;
-  int* counter;                // device work counter: zero between launches (the kernels set it back)
+  unsigned* counter;           // device work counter: zero between launches (see next_item), one per launch shape
   const float2* tw;            // e^{-2 pi i k / Mmax}, k < Mmax
   int Mmax;
   int H;                       // half tap count (taps = 2H)

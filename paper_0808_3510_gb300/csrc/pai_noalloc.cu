@@ -130,7 +130,7 @@ extern "C" pai_status pai_spectrum_rows_noalloc(const pai_geometry* g_in, const 
   L.problems = reinterpret_cast<const RowProblem*>(base + o_prob);
   L.items = reinterpret_cast<const WorkItem*>(base + o_items);
   L.nitems = nitems;
-  L.counter = reinterpret_cast<int*>(base + o_count);
+  L.counter = reinterpret_cast<unsigned*>(base + o_count);
   L.tw = reinterpret_cast<const float2*>(base + o_tw);
   L.Mmax = pp.M;
   L.H = pp.H;

@@ -1081,17 +1081,19 @@ __device__ __forceinline__ void gather_row_z(const RowProblem& P, const WindowPo
 // The next work item for the whole CTA (dynamic scheduling).  A CTA's first
 // item is its block index (the grid is never larger than the item list), so
 // no CTA waits for a counter before it starts; every further item costs one
-// atomicAdd.  The CTAs fetch exactly nitems times in all (nitems - gridDim.x
-// items and one empty fetch each), so the CTA that draws the last ticket sets
-// the counter back to zero for the next launch: no memset runs before the
-// kernel (0.9 us plus a launch gap of about 1 us per pass before).
+// atomic.  The CTAs fetch exactly nitems times in all (nitems - gridDim.x
+// items and one empty fetch each), and the atomic counts modulo nitems, so it
+// leaves zero for the next launch: no memset runs before the kernel (0.9 us plus
+// a launch gap of about 1 us per pass before).  The same holds for launches of
+// one shape that overlap (calls on one plan that nobody ordered): every nitems
+// tickets hold one empty one per CTA of a launch, so the counter is at zero again
+// when the last of them ends, whatever their order.  (Set back by a store of its
+// own, it could lose tickets drawn in between, and a later call left out rows.)
 __device__ __forceinline__ int next_item(const RowLaunch& L, int* s_item) {
   if (L.nitems <= (int)gridDim.x) return L.nitems;  // one item per CTA: the counter is not used
   __syncthreads();
   if (threadIdx.x == 0) {
-    const int ticket = atomicAdd(L.counter, 1);
-    if (ticket == L.nitems - 1) *L.counter = 0;
-    *s_item = (int)gridDim.x + ticket;
+    *s_item = (int)(gridDim.x + atomicInc(L.counter, (unsigned)(L.nitems - 1)));
   }
   __syncthreads();
   return *s_item;

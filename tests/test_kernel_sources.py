@@ -1,6 +1,7 @@
 """Rules the CUDA sources keep, read from the sources themselves (what they guard against shows on a GPU only now and
 then, or not with today's compiler)."""
 import os
+import random
 import re
 
 import pytest
@@ -41,3 +42,26 @@ def test_dynamic_shared_memory_is_aligned_for_16_byte_cells(name):
     """Row slots hold 16-byte cells and node records at offsets that are multiples of 16: the base has to be one."""
     for m in re.finditer(r"extern\s+__shared__([^;]*);", _code(name)):
         assert "__align__(16)" in m.group(1), f"{name}: extern __shared__{m.group(1)}"
+
+
+@pytest.mark.parametrize("nitems,ctas,launches", [(2, 1, 1), (40, 7, 1), (2, 1, 2), (5, 4, 2), (40, 7, 2), (40, 7, 3), (301, 152, 2)])
+def test_work_counter_is_zero_after_overlapping_launches(nitems, ctas, launches):
+    """The row kernels draw work items from a counter that no launch sets beforehand: it has to be zero after every
+    launch, and after launches that overlapped in any order, or the next call would leave out rows."""
+    code = _code("pai_row_kernels.cuh")
+    uses = re.findall(r"\bL\.counter\b[^;]*", code)
+    assert len(uses) == 1 and uses[0].startswith("L.counter, (unsigned)(L.nitems - 1))")
+    assert "gridDim.x + atomicInc(L.counter" in code
+    for seed in range(20):
+        rng = random.Random(seed)
+        counter, done = 0, [set(range(ctas)) for _ in range(launches)]  # the first items are the block indices
+        running = [(k, c) for k in range(launches) for c in range(ctas)]
+        while running:
+            i = rng.randrange(len(running))
+            ticket, counter = counter, 0 if counter >= nitems - 1 else counter + 1  # atomicInc
+            if ctas + ticket < nitems:
+                done[running[i][0]].add(ctas + ticket)
+            else:
+                running.pop(i)
+        assert counter == 0
+        assert launches > 1 or done[0] == set(range(nitems))
