@@ -115,9 +115,9 @@ typedef struct {
   int rows;               /* lateral-frequency rows processed per call          */
   long long nodes;        /* nodes evaluated per call (sum over the batch)      */
   size_t workspace_bytes; /* device bytes owned by the plan                     */
-  int uses_graph;         /* 1 if reconstructions or adjoints replay a captured
-                             CUDA graph (plans that run cuFFT, batches, all but
-                             large problems)                                   */
+  int uses_graph;         /* 1 if reconstructions or adjoints may replay a
+                             captured CUDA graph (plans that run cuFFT, batches,
+                             all but large problems)                           */
   int library_ffts;       /* bit 0: pai_reconstruct runs every stage on the
                              library's own kernels (power-of-two sizes, chosen
                              by the tuner), else its inverse uses cuFFT; bit 1:

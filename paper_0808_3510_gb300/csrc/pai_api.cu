@@ -15,6 +15,7 @@
 #include <cufft.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdint>
@@ -24,6 +25,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "../../include/pai.h"
@@ -34,6 +36,10 @@ using namespace pai;
 namespace {
 
 constexpr double kPi = 3.14159265358979323846;
+// Timed reconstruction plus adjoint from which all calls launch directly (see
+// pai_plan_s::graphed): the 212 us a direct gradient step takes the host, and the
+// 10 us by which the tuner's two passes read longer than repeated ones.
+constexpr float kDirectMs = 0.22f;
 
 struct ProblemHost {
   pai_geometry g;
@@ -93,14 +99,22 @@ struct pai_plan_s {
   // stream they follow the previous call closer than graph replays do (2048x4096:
   // 97.7 us a pass against 104.2 with a graph, its adjoint 138 and 144), but they
   // take the host 20 to 25 us instead of 10, and about 50 us more in a gradient
-  // step, whose adjoint runs on autograd's thread (128^3: 209 against 156 us a
-  // step, all of it host time).  So they are direct where the kernels of such a
-  // step outlast its host time of about 200 us: from some ten million samples and
-  // voxels.  Calls of many cuFFT launches and of batches replay a graph.
-  bool graphed(bool adjoint) const {
+  // step, whose adjoint runs on autograd's thread (209 to 216 against 156 us a
+  // step, all of it host time).  So from ten million samples and voxels calls that
+  // follow each other on one thread are direct; calls that change threads (hop:
+  // a gradient step's) are direct only where the tuner timed a reconstruction and
+  // its adjoint at kDirectMs together or more, so that the kernels of such a step
+  // outlast its host time.  (By size alone, 128x256x256 at 64 depths, 167 us of
+  // kernels, took 213 to 216 us a gradient step directly and takes 174 now; 200
+  // with the graphs and kernels of before.)  Calls of many cuFFT launches and of
+  // batches replay a graph.
+  bool slow_step = false;  // the tuner timed a step at kDirectMs or more
+  bool graphed(bool adjoint, bool hop) const {
     if (!use_graph) return false;
-    return probs.size() > 1 || !(adjoint ? zf_adj : zf) || data_total + img_total < ((size_t)10 << 20);
+    if (probs.size() > 1 || !(adjoint ? zf_adj : zf)) return true;
+    return !slow_step && (hop || data_total + img_total < ((size_t)10 << 20));
   }
+  std::atomic<std::thread::id> caller{};  // the thread of the last call
   WindowPoly poly{};
   double beta = 0, pred_err = 0, fit_err = 0;
   size_t data_total = 0, img_total = 0;
@@ -563,7 +577,8 @@ pai_status run(pai_plan_s* P, const void* in, void* out, bool adjoint) {
   cudaSetDevice(P->device);
   pai_status st = in_callers_capture(P) ? PAI_ERR_CUDA : PAI_OK;
   GraphEntry* hit = nullptr;
-  bool direct = !P->graphed(adjoint);
+  const std::thread::id me = std::this_thread::get_id(), before = P->caller.exchange(me, std::memory_order_relaxed);
+  bool direct = !P->graphed(adjoint, before != me && before != std::thread::id());
   if (st == PAI_OK && !direct) {
     for (auto& ge : P->graphs)
       if (ge.in == in && ge.out == out && ge.adjoint == adjoint) hit = &ge;
@@ -628,7 +643,7 @@ struct Wisdom {
   int H = 0;
   std::vector<int> M;  // empty: the window was not tuned
   int threads = 0, threads_adj = 0, spread_tuned = 1, spread_det = 0;
-  bool zf = false, zf_adj = false;
+  bool zf = false, zf_adj = false, slow_step = false;
   std::string log;
 };
 std::mutex g_wisdom_mutex;
@@ -1366,6 +1381,7 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
   if (P->zf && tune && have_wis) {
     P->zf = wis.zf;
     P->zf_adj = wis.zf_adj;
+    P->slow_step = wis.slow_step;
   } else if (P->zf && tune) {
     float* d_in = nullptr;
     float* d_out = nullptr;
@@ -1398,6 +1414,8 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
         else (variant == 0 ? ms_zf : ms_cufft) = best;
       }
       P->zf_adj = adj_zf <= adj_cufft;
+      const float step = std::min(ms_zf, ms_cufft) + std::min(adj_zf, adj_cufft);
+      P->slow_step = step >= kDirectMs && step < 1e29f;
       std::snprintf(logline, sizeof logline,
                     "pipeline: forward pass %.4f ms with the library's transforms, %.4f ms with cuFFT; adjoint "
                     "%.4f / %.4f ms\n", ms_zf, ms_cufft, adj_zf, adj_cufft);
@@ -1452,6 +1470,7 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     w.spread_det = P->spread_det;
     w.zf = P->zf;
     w.zf_adj = P->zf_adj;
+    w.slow_step = P->slow_step;
     w.log = P->tune_log;
     std::lock_guard<std::mutex> lock(g_wisdom_mutex);
     g_wisdom.emplace(wkey, std::move(w));
@@ -1707,7 +1726,7 @@ pai_status pai_get_info(pai_plan_t plan, pai_plan_info* info) {
   info->rows = plan->rows_total;
   info->nodes = plan->nodes;
   info->workspace_bytes = plan->ws_bytes;
-  info->uses_graph = plan->graphed(false) || plan->graphed(true) ? 1 : 0;
+  info->uses_graph = plan->graphed(false, true) || plan->graphed(true, true) ? 1 : 0;
   info->library_ffts = (plan->zf ? 1 : 0) | (plan->zf_adj ? 2 : 0);
   return PAI_OK;
 }
