@@ -52,7 +52,12 @@ typedef enum {
   PAI_ERR_UNSUPPORTED = 2,  /* valid but outside what this build implements  */
   PAI_ERR_OOM = 3,          /* device or host allocation failed              */
   PAI_ERR_CUDA = 4,         /* a CUDA runtime call or kernel launch failed, or
-                               the plan's stream is being captured           */
+                               the plan's stream is being captured (calls on
+                               host memory, pai_profile_stages and, unless the
+                               plan was made with PAI_USE_GRAPH=0,
+                               pai_reconstruct, pai_adjoint and
+                               pai_forward_model; refused before they do
+                               anything)                                     */
   PAI_ERR_CUFFT = 5,        /* a cuFFT call failed                           */
   PAI_ERR_TIMEOUT = 6       /* a bounded device-side wait gave up            */
 } pai_status;
@@ -175,7 +180,9 @@ pai_status pai_adjoint(pai_plan_t plan, const float* d_h, float* d_pbar);
  * d_fhat: device, interleaved complex64, [nx][ny][nz/2+1] per problem
  * (half spectrum in depth, full lateral spectrum), including the factor
  * 1/(nx*ny*nz) of the inverse FFT.  Entry l = nz/2 holds the mean of the two
- * Nyquist nodes (the real part of the inverse DFT depends only on it).        */
+ * Nyquist nodes (the real part of the inverse DFT depends only on it).  May be
+ * captured into a caller's graph, which must not be replayed after
+ * pai_destroy (it uses the plan's memory).                                    */
 pai_status pai_spectrum(pai_plan_t plan, const float* d_p, float* d_fhat);
 
 /* End-to-end reconstruction from HOST memory: copies h_p to the device,
@@ -359,7 +366,7 @@ pai_status pai_forward_box(pai_plan_t plan, int* bx, int* by, int* bz);
  * (device FP32, contiguous).  d_in == d_out (in place) touches only the
  * samples whose weight differs from one; partially overlapping buffers are
  * not allowed.  PAI_ERR_INVALID_ARG without a cutoff set.  Asynchronous on
- * the plan's stream.                                                         */
+ * the plan's stream; may be captured as pai_spectrum.                        */
 pai_status pai_cutoff_table(int dim, double eps, double* table, int capacity, int* R);
 pai_status pai_set_cutoff(pai_plan_t plan, double eps);
 pai_status pai_cutoff(pai_plan_t plan, const float* d_in, float* d_out);

@@ -554,12 +554,14 @@ pai_status enqueue_adjoint(pai_plan_s* P, const float* d_h, float* d_pbar, cudaS
   return enqueue_last(P, d_pbar, s, true);
 }
 
-// A plan's calls are not part of a caller's stream capture (PAI_USE_GRAPH=0
-// plans excepted): a graph of the caller's would hold the plan's workspace beyond
-// pai_destroy.  Refused before anything is launched, so that the capture stays
-// whole, and alike for calls that launch directly and calls that replay a graph.
-bool in_callers_capture(pai_plan_s* P) {
-  if (!P->use_graph) return false;
+// Whether a caller is capturing the plan's stream.  Calls that cannot be part of
+// a capture are refused before they do anything, so that the capture stays whole:
+// host-memory calls and profiling, which wait for the device or for streams
+// outside the capture, and, unless the plan was made with PAI_USE_GRAPH=0,
+// reconstructions, adjoints and forward models, alike whether they launch
+// directly or replay a graph.  (pai_spectrum and pai_cutoff are captured; such a
+// graph uses the plan's memory and must not outlive it.)
+bool capturing(pai_plan_s* P) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(P->stream, &cs) != cudaSuccess) {
     cudaGetLastError();
@@ -575,7 +577,7 @@ pai_status run(pai_plan_s* P, const void* in, void* out, bool adjoint) {
   // CUDA call yet (autograd's backward threads) this makes its context current,
   // which a direct cuFFT execution needs
   cudaSetDevice(P->device);
-  pai_status st = in_callers_capture(P) ? PAI_ERR_CUDA : PAI_OK;
+  pai_status st = P->use_graph && capturing(P) ? PAI_ERR_CUDA : PAI_OK;
   GraphEntry* hit = nullptr;
   const std::thread::id me = std::this_thread::get_id(), before = P->caller.exchange(me, std::memory_order_relaxed);
   bool direct = !P->graphed(adjoint, before != me && before != std::thread::id());
@@ -1557,8 +1559,8 @@ pai_status pai_reconstruct_host(pai_plan_t plan, const float* h_p, float* h_f) {
   int prev = 0;
   cudaGetDevice(&prev);
   if (prev != plan->device) cudaSetDevice(plan->device);
-  pai_status st = PAI_OK;
-  if (!plan->d_stage_in || !plan->d_stage_out) {
+  pai_status st = capturing(plan) ? PAI_ERR_CUDA : PAI_OK;
+  if (st == PAI_OK && (!plan->d_stage_in || !plan->d_stage_out)) {
     st = plan_malloc(plan, (void**)&plan->d_stage_in, plan->data_total * sizeof(float));
     if (st == PAI_OK) st = plan_malloc(plan, (void**)&plan->d_stage_out, plan->img_total * sizeof(float));
     if (st != PAI_OK) {
@@ -1592,8 +1594,8 @@ pai_status pai_reconstruct_host_async(pai_plan_t plan, const float* h_p, float* 
   int prev = 0;
   cudaGetDevice(&prev);
   if (prev != plan->device) cudaSetDevice(plan->device);
-  pai_status st = PAI_OK;
-  if (!plan->pipe_ready) {
+  pai_status st = capturing(plan) ? PAI_ERR_CUDA : PAI_OK;
+  if (st == PAI_OK && !plan->pipe_ready) {
     if (!plan->s_up) st = cuda_status(cudaStreamCreateWithFlags(&plan->s_up, cudaStreamNonBlocking));
     if (st == PAI_OK && !plan->s_down) st = cuda_status(cudaStreamCreateWithFlags(&plan->s_down, cudaStreamNonBlocking));
     for (int k = 0; k < 2 && st == PAI_OK; ++k) {
@@ -1652,7 +1654,7 @@ pai_status pai_profile_stages(pai_plan_t plan, const float* d_in, float* d_out, 
   cudaGetDevice(&prev);
   if (prev != plan->device) cudaSetDevice(plan->device);
   cudaEvent_t ev[4];
-  pai_status st = PAI_OK;
+  pai_status st = capturing(plan) ? PAI_ERR_CUDA : PAI_OK;
   int made = 0;
   for (; made < 4 && st == PAI_OK; ++made) st = cuda_status(cudaEventCreate(&ev[made]));
   double acc[3] = {0, 0, 0};
@@ -1821,7 +1823,7 @@ pai_status pai_forward_model(pai_plan_t plan, const float* d_f, float* d_p) {
   const int ny = gi.dim == 3 ? gi.ny : 1;
   // plain launches, not a graph kept per pointer pair: four to six kernels of a
   // call that takes longer than their launches, and no capture on new buffers
-  pai_status st = in_callers_capture(plan) ? PAI_ERR_CUDA : PAI_OK;
+  pai_status st = plan->use_graph && capturing(plan) ? PAI_ERR_CUDA : PAI_OK;
   if (st == PAI_OK) st = enqueue_adjoint(plan, d_f, d_p, plan->stream);
   if (st == PAI_OK) plan->own_kernels += plan->own_kernels_per_adj;
   if (st == PAI_OK && plan->d_cut) {
