@@ -539,11 +539,10 @@ class ForwardModel:
         return _tuning_log(self._lib, self._h)
 
     def profile_stages(self, reps: int = 10):
-        """Mean device ms of (image-side transforms, forward-model row kernel, lateral inverse) on the box."""
-        bx, by, bz = self.box
+        """Mean device ms of (image-side transforms, forward-model row kernel, lateral inverse)."""
         g = self.geom
-        x = torch.zeros(bx * by * bz, device=self.device, dtype=torch.float32)
-        y = torch.empty(bx * by * g.nt, device=self.device, dtype=torch.float32)
+        x = torch.zeros(_shape(g, g.nz), device=self.device, dtype=torch.float32)
+        y = torch.empty(_shape(g, g.nt), device=self.device, dtype=torch.float32)
         ms = (ctypes.c_double * 3)()
         _check(self._lib.pai_profile_stages(self._h, ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(y.data_ptr()),
                                             int(reps), 1, ms), "pai_profile_stages")

@@ -364,6 +364,7 @@ void release(pai_plan_s* P) {
 pai_status set_fft_streams(pai_plan_s* P, cudaStream_t s) {
   if (P->nbranch > 1) return PAI_OK;  // batched plans keep their plans on the branch streams
   for (auto& p : P->probs) {
+    if (!p.have_plans) continue;  // forward models
     PAI_FFT(cufftSetStream(p.lat_r2c, s));
     PAI_FFT(cufftSetStream(p.lat_c2r, s));
     PAI_FFT(cufftSetStream(p.img_c2r, s));
@@ -962,8 +963,10 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
   }
 
   // ---- cuFFT ----------------------------------------------------------------
+  // (a forward model runs none: its box is transformed by the library's kernels)
   size_t work = 0;
-  for (auto& p : P->probs) PAI_TRY(make_cufft_plans(P, p, work));
+  if (!qmode)
+    for (auto& p : P->probs) PAI_TRY(make_cufft_plans(P, p, work));
   P->cufft_work = work;
   P->nbranch = std::min(count, 4);  // measured on the 64-problem batch: 4 beat 2, 6, 8, 16, 32
   if (P->nbranch > 1) {
