@@ -122,7 +122,7 @@ typedef struct {
   size_t workspace_bytes; /* device bytes owned by the plan                     */
   int uses_graph;         /* 1 if reconstructions or adjoints may replay a
                              captured CUDA graph (plans that run cuFFT, batches,
-                             all but large problems)                           */
+                             all but large problems; forward models never do)  */
   int library_ffts;       /* bit 0: pai_reconstruct runs every stage on the
                              library's own kernels (power-of-two sizes, chosen
                              by the tuner), else its inverse uses cuFFT; bit 1:

@@ -48,3 +48,8 @@ def test_same_bits_on_one_thread_and_on_changing_threads(pai):
     for _ in range(5):
         (g,) = torch.autograd.grad(pai.PAIRecon.apply(x, plan), x, h)
         assert torch.equal(g, a)
+
+
+def test_forward_models_never_replay_graphs(pai):
+    model = pai.ForwardModel(dict(dim=2, nx=64, nt=128, nz=64, dx=1.0, dt=1.0, c=1.0, dz=1.0))
+    assert model.info["uses_graph"] == 0
