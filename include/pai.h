@@ -219,7 +219,11 @@ pai_status pai_host_wait(pai_plan_t plan);
  * d_in / d_out as for pai_reconstruct / pai_adjoint; ms: host, 3 doubles.   */
 pai_status pai_profile_stages(pai_plan_t plan, const float* d_in, float* d_out, int reps, int adjoint, double* ms);
 
-/* Change the stream later calls are enqueued on (cudaStream_t or NULL).     */
+/* Change the stream later calls are enqueued on (cudaStream_t or NULL).  A
+ * plan's calls share its workspace and are ordered by their stream only: the
+ * caller makes the new stream wait for the calls still in flight on the old
+ * one (an event), or calls that overlap spoil each other's results.  The old
+ * stream is not touched and may be gone already.                             */
 pai_status pai_set_stream(pai_plan_t plan, void* cuda_stream);
 
 /* Spread of pai_adjoint and pai_forward_model (the transpose of the window

@@ -272,7 +272,9 @@ class Plan:
     ``Plan(g)`` wraps ``pai_plan``; ``Plan([g0, g1, ...])`` wraps
     ``pai_plan_batched`` (inputs and outputs are then flat concatenations).
     The plan lives on the current CUDA device; calls run on torch's current
-    stream.
+    stream.  They share the plan's workspace: a call on another stream than the
+    one before has to be ordered behind it (``new.wait_stream(old)``), and one
+    plan is used by one thread at a time.
     """
 
     def __init__(self, geoms, stream: Optional[torch.cuda.Stream] = None, overrides: Optional[dict] = None):
@@ -467,7 +469,7 @@ class ForwardModel:
     """Discrete forward model (``pai_forward_plan`` / ``pai_forward_model``): detector
     data of an initial pressure on the image grid, the wave equation solved
     exactly for its trigonometric interpolant in a zero-padded periodic box.
-    Calls run on torch's current stream."""
+    Calls run on torch's current stream, ordered as a :class:`Plan`'s."""
 
     def __init__(self, g, stream: Optional[torch.cuda.Stream] = None, cutoff: Optional[float] = None):
         lib = load_library()
@@ -590,7 +592,9 @@ def _geometry_key(gg: Geometry):
 def cached_plan(g) -> Plan:
     """A single-problem :class:`Plan` for geometry ``g`` on the current device,
     created on first use and kept (least recently used first out, at most
-    eight; a dropped plan is destroyed when its last user lets go of it)."""
+    eight; a dropped plan is destroyed when its last user lets go of it).  All
+    users of a geometry share it: order their streams as for any :class:`Plan`,
+    or make plans of their own."""
     gg = geometry(g)
     key = (_geometry_key(gg), torch.cuda.current_device())
     with _plan_cache_lock:
