@@ -75,7 +75,7 @@ struct pai_plan_s {
   int H = 0, Mmax = 0, threads = 512, ctas = 0, ctas_adj = 0, fft_region = 0;
   int threads_adj = 512, fft_region_adj = 0;  // the adjoint row kernel's own CTA shape
   int TW = 0;  // twiddle table length (power of two >= every FFT length the plan runs)
-  int chunk = 128, bin_offset = 0, bin_slot = 0;  // adjoint sorted-bin spread
+  int chunk = 128;                                  // adjoint, spread by tap phases: nodes per chunk
   int method = PAI_METHOD_KB;                       // PAI_METHOD_*, shared by the batch
   int spread_mode = 1;                              // adjoint spread (RowLaunch::spread_mode): atomics
   int spread_tuned = 1;                             // the faster spread found when the plan was built
@@ -384,8 +384,6 @@ RowLaunch make_launch(pai_plan_s* P, bool adjoint) {
   L.H = P->H;
   L.fft_region = adjoint ? P->fft_region_adj : P->fft_region;
   L.chunk = P->chunk;
-  L.bin_offset = P->bin_offset;
-  L.bin_slot = P->bin_slot;
   L.spread_mode = P->spread_mode;
   if (adjoint && P->spread_mode == 4) {
     L.items = P->d_items_model;
@@ -1067,9 +1065,7 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     }
     const int span_cap = std::max(1, (int)((m_min - 2 * P->H - 1) / (std::ceil(gap) + 1)));
     P->chunk = std::max(1, std::min(tpr_min, span_cap));
-    P->bin_slot = 0;
-    P->bin_offset = (int)(region + (size_t)node_cap * sizeof(float4));
-    P->smem_adj = (size_t)P->bin_offset;
+    P->smem_adj = region + (size_t)node_cap * sizeof(float4);
     if (P->smem_adj > (size_t)smem_optin) return PAI_ERR_UNSUPPORTED;
     const int occ_a = row_kernel_max_ctas_per_sm(1, T, P->smem_adj, P->H, P->zf);
     if (occ_a < 1) return PAI_ERR_UNSUPPORTED;

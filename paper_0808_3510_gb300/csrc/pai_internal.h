@@ -107,7 +107,6 @@ struct RowProblem {
   float wscale;            // 2 c dt/dz * B / (n1 n2 nz): W = wscale * kz / x
   float nt_over_M;         // for the node phase
   int mshift;              // log2(M)
-  int nzshift;             // log2(nz) when nz is a power of two, else 0
   int method;              // PAI_METHOD_*
   int qmode;               // adjoint kernel evaluates the discrete forward model (depth-row layout only)
   int zstride;             // depth-row layout: complex values from one row to the next (nz; in qmode
@@ -135,10 +134,7 @@ struct RowLaunch {
   int Mmax;
   int H;                       // half tap count (taps = 2H)
   int fft_region;              // complex values of shared memory used by the row slots (adjoint: nodes follow)
-  // adjoint only: sorted-bin spread buffers
-  int chunk;                   // nodes per bin chunk
-  int bin_offset;              // bytes from the start of dynamic shared memory to the bins
-  int bin_slot;                // bytes of bins per row slot: chunk * (2H+1) complex, 16-aligned
+  int chunk;                   // adjoint, spread mode 0: nodes per chunk
   int spread_mode;             // adjoint spread: 0 tap phases (deterministic), 1 shared-memory atomics per
                                // node, 2 shared-memory atomics per run of nodes with equal j0, 3 node pairs
                                // into band grids (deterministic; windowed methods; not qmode), 4 the
@@ -227,6 +223,7 @@ size_t row_fft_region_bytes(int threads, int M);
 bool lateral_supported(int L, int C);
 // n (0: L): only the first n of the L points of the axis exist on the side named real (c2c: on the input of the
 // forward, the output of the inverse transform): A[outer][n][C]; the others are zeros (input) or not wanted (output).
+// c2c in place: with n = L, or outer = 1 (a point then lies at the same place on both sides).
 cudaError_t launch_lateral_r2c(const float* in, float2* out, int L, int C, int outer, const float2* tw, int twstride,
                                cudaStream_t s, bool pdl, int n = 0);
 cudaError_t launch_lateral_c2r(const float2* in, float* out, int L, int C, int outer, const float2* tw, int twstride,

@@ -240,9 +240,11 @@ cudaError_t launch_lateral_c2r(const float2* in, float* out, int L, int C, int o
   return lat_any<kLatC2R>(in, out, L, C, outer, tw, twstride, s, pdl, n);
 }
 
-// out[o][k][c] = sum_x e^{-+2 pi i k x / L} in[o][x][c]; in place allowed when not pruned (each CTA owns its columns).
+// out[o][k][c] = sum_x e^{-+2 pi i k x / L} in[o][x][c]; in place where a point lies at the same place on both sides
+// (each CTA owns its columns): not pruned, or outer = 1.
 cudaError_t launch_lateral_c2c(const float2* in, float2* out, int L, int C, int outer, bool inverse, const float2* tw,
                                int twstride, cudaStream_t s, bool pdl, int n) {
+  if (in == out && n > 0 && n < L && outer != 1) return cudaErrorInvalidValue;
   if (inverse) return lat_any<kLatC2CInv>(in, out, L, C, outer, tw, twstride, s, pdl, n);
   return lat_any<kLatC2C>(in, out, L, C, outer, tw, twstride, s, pdl, n);
 }

@@ -846,23 +846,6 @@ __device__ __forceinline__ float2 node_phase(int j0, float fr, int nt, int M, fl
   return make_float2(c1 * c2 - s1 * s2, s1 * c2 + c1 * s2);
 }
 
-// All 2H tap weights of a node with fraction fr (constant-bank coefficients).
-template <int H>
-__device__ __forceinline__ void tap_weights(const WindowPoly& W, float fr, float (&w)[2 * H]) {
-  const float z = fr - 0.5f, z2 = z * z;
-#pragma unroll
-  for (int p = 0; p < H; ++p) {
-    float E = W.ce[p][kHalfCoef - 1], O = W.co[p][kHalfCoef - 1];
-#pragma unroll
-    for (int e = kHalfCoef - 2; e >= 0; --e) {
-      E = fmaf(E, z2, W.ce[p][e]);
-      O = fmaf(O, z2, W.co[p][e]);
-    }
-    w[p] = fmaf(z, O, E);
-    w[2 * H - 1 - p] = fmaf(-z, O, E);
-  }
-}
-
 // P(nu) = e^{-i pi nu} sum_t w_t G[(j0 + t) mod M], t = -H+1..H   (Eq. nufft-a).
 // U is the flat spectrum with ghost cells: the 2H taps are U[b .. b+2H-1],
 // b = (j0 - H + 1) mod M.  Weights are formed pair by pair (tap it and its
@@ -1167,10 +1150,6 @@ __device__ __forceinline__ float interp_tap_weight(int method, int t, float fr) 
   return (t == 1) ? 1.0f - fr : (t == 2 ? fr : 0.0f);
 }
 
-__device__ __forceinline__ int floor_div(int a, int b) {  // b > 0
-  return (a >= 0) ? a / b : -((-a + b - 1) / b);
-}
-
 // Where a row's node pairs come from.
 struct PairSrc {
   const float2* a;  // ZF: the row's depth spectrum; else the +k line of the half spectrum
@@ -1457,7 +1436,7 @@ struct BandPart {
   // a pass over two nodes adds (zeros) up to kReach cells beyond the second one's last
   static constexpr int kReach = 2;
   static constexpr int kSpill = 2 * H + 4 + kReach;  // at most 32
-  int nw, wa, w;       // warps, warps with nodes, this warp
+  int nw, wa, w;       // warps, warps with nodes (as few as hold 32 each, at most nw; np is shared evenly), this warp
   int gw, l;           // lanes per row in a warp, this lane's place
   int n0, n1;          // this warp's nodes
   int lo_w, hi_prev;   // first cell of this warp's nodes, last cell of its predecessor's
@@ -1476,7 +1455,7 @@ __device__ __forceinline__ void band_begin(BandPart<H>& b, Band& band, char* slo
   b.gw = threads < 32 ? threads : 32;
   b.w = threads > 32 ? lane >> 5 : 0;
   b.l = lane & (b.gw - 1);
-  b.wa = min(b.nw, (np + 31) >> 5);  // warps with a full chunk of nodes each
+  b.wa = min(b.nw, (np + 31) >> 5);
   const bool on = b.w < b.wa;
   b.n0 = on ? np * b.w / b.wa : np;
   b.n1 = on ? np * (b.w + 1) / b.wa : np;

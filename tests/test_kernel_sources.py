@@ -65,3 +65,9 @@ def test_work_counter_is_zero_after_overlapping_launches(nitems, ctas, launches)
                 running.pop(i)
         assert counter == 0
         assert launches > 1 or done[0] == set(range(nitems))
+
+
+def test_every_device_function_is_used():
+    code = "".join(_code(f) for f in sorted(os.listdir(CSRC)) if f.endswith((".cu", ".cuh", ".h", ".cpp")))
+    for name in set(re.findall(r"__device__\s+__forceinline__\s+[\w:<>, ]*?[&*]?\s(\w+)\(", code)):
+        assert len(re.findall(rf"\b{name}\b", code)) > 1, name
