@@ -244,7 +244,9 @@ pai_status pai_set_stream(pai_plan_t plan, void* cuda_stream);
  * that applies and keeps the fastest (the environment variable PAI_SPREAD
  * forces one by the names above; "pairs_atomic", an earlier variant, selects
  * pairs).  pai_forward_model runs a row kernel of its own, bit-identical on
- * repeated calls, unless one of the first three is forced.
+ * repeated calls, unless one of the first three is forced, its rows do not fit
+ * or the window's predicted error exceeds 1e-6 (truncated sinc; Kaiser-Bessel
+ * with fewer than 8 taps at oversampling 2): then one of the spreads above.
  * deterministic = 1: the faster of tap and pairs; deterministic = 0: back to
  * the plan's choice.  pai_reconstruct is deterministic either way.  Waits for
  * the plan's stream and drops the plan's captured CUDA graphs (they are

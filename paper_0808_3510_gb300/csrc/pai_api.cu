@@ -40,6 +40,8 @@ constexpr double kPi = 3.14159265358979323846;
 // pai_plan_s::graphed): the 212 us a direct gradient step takes the host, and the
 // 10 us by which the tuner's two passes read longer than repeated ones.
 constexpr float kDirectMs = 0.22f;
+// Predicted window error up to which a forward model runs its own row kernel.
+constexpr double kModelErr = 1e-6;
 
 struct ProblemHost {
   pai_geometry g;
@@ -390,6 +392,7 @@ RowLaunch make_launch(pai_plan_s* P, bool adjoint) {
     L.nitems = P->nitems_model;
     L.model_pair = P->probs[0].g.dim == 3 ? 1 : 0;
   }
+  L.qmode = P->qmode ? 1 : 0;
   L.paired = !adjoint && P->any_paired ? 1 : 0;
   L.pdl = P->pdl();
   return L;
@@ -1072,14 +1075,14 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     // spread mode 3 (node pairs into band grids): windowed methods, as long as
     // the bands fit in shared memory (up to c dt / dz = 3.4 at M = 8192, 1.7 at
     // 16384, far more for shorter rows)
-    P->pairs_ok = !qmode && !method_interp(P->method) && std::getenv("PAI_NO_PAIRS") == nullptr;
+    P->pairs_ok = !method_interp(P->method) && std::getenv("PAI_NO_PAIRS") == nullptr;
     P->smem_adj3 = 0;
     for (int i = 0; i < count; ++i)
       P->smem_adj3 = std::max(P->smem_adj3, (size_t)(T / P->probs[i].tpr) * (size_t)rp[i].band_slot * sizeof(float2));
     if (P->smem_adj3 > (size_t)smem_optin) P->pairs_ok = false;
     P->ctas_adj3 = 0;
     if (P->pairs_ok) {
-      const int occ3 = row_kernel_max_ctas_per_sm(2, T, P->smem_adj3, P->H, P->zf);
+      const int occ3 = row_kernel_max_ctas_per_sm(qmode ? 6 : 2, T, P->smem_adj3, P->H, P->zf);
       if (occ3 < 1) P->pairs_ok = false;
       P->ctas_adj3 = occ3 * sms;
     }
@@ -1302,8 +1305,13 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
   if (env_mode == 4) env_mode = P->pairs_ok || qmode ? 3 : 1;
   if (env_mode == 3 && !P->pairs_ok && !qmode) env_mode = 0;
   // forward models run their own row kernel (see row_model_kernel) unless it
-  // does not fit or one of the list spreads is forced; its CTA size is timed
-  if (qmode && (env_mode < 0 || env_mode == 3)) {
+  // does not fit or one of the list spreads is forced; its CTA size is timed.
+  // It evaluates the window over the doubled interval, so that the window's error
+  // falls on other samples than with the node pairs: only where that error is below
+  // rounding (Kaiser-Bessel from 8 taps at oversampling 2) are the results the
+  // same.  Truncated sinc and shorter windows keep the node pairs (4 taps: errors
+  // of up to 1.9 times theirs otherwise).
+  if (qmode && P->pred_err <= kModelErr && (env_mode < 0 || env_mode == 3)) {
     const int tpu = (P->probs[0].g.dim == 3 ? 2 : 1) * P->probs[0].tpr;
     int best_T = 0;
     float best_ms = 1e30f;
@@ -1334,6 +1342,7 @@ pai_status build_plan(const pai_geometry* gs, int count, void* stream, pai_plan_
     P->model_ok = best_T > 0 && finish_shape_model(best_T) == PAI_OK;
     env_mode = P->model_ok ? 4 : -1;
   }
+  if (env_mode == 3 && !P->pairs_ok) env_mode = -1;
   P->spread_det = P->model_ok ? 4 : P->pairs_ok ? 3 : 0;
   if (env_mode >= 0) {
     P->spread_tuned = env_mode;

@@ -137,9 +137,10 @@ struct RowLaunch {
   int chunk;                   // adjoint, spread mode 0: nodes per chunk
   int spread_mode;             // adjoint spread: 0 tap phases (deterministic), 1 shared-memory atomics per
                                // node, 2 shared-memory atomics per run of nodes with equal j0, 3 node pairs
-                               // into band grids (deterministic; windowed methods; not qmode), 4 the
+                               // into band grids (deterministic; windowed methods), 4 the
                                // forward-model row kernel (deterministic; qmode only)
   int model_pair;              // spread mode 4: units of two rows (3-D)
+  int qmode;                   // adjoint launch of a forward-model plan
   bool pdl;                    // launch as a programmatic dependent (launch_kernel)
   int paired;                  // forward: some problem is in the paired layout (RowProblem::paired)
 };
@@ -238,7 +239,8 @@ cudaError_t launch_rows_c2c(float2* data, int L, int rows, bool inverse, const f
 cudaError_t launch_rows_fold(const float2* in, int n, float2* out, int L, int rows, const float2* tw, int twstride,
                              cudaStream_t s, bool pdl);
 // kind: 0 forward row kernel, 1 adjoint row kernel, 2 adjoint row kernel with the pair spread, 3 forward row
-// kernel for launches with problems in the paired layout, 4 forward-model row kernel, 5 the same in units of two rows
+// kernel for launches with problems in the paired layout, 4 forward-model row kernel, 5 the same in units of two
+// rows, 6 forward model by node pairs
 int row_kernel_max_ctas_per_sm(int kind, int threads, size_t smem, int H, bool zf = false);
 
 // Data cutoff w_cut (pai_cutoff.cu).  R = ceil(sqrt(eps)); the table holds

@@ -43,6 +43,7 @@ static cudaError_t adj_h(const RowLaunch& L, const WindowPoly& w, int threads, i
   if (L.spread_mode == 4)
     return L.model_pair ? launch_k(row_model_kernel<H, true>, L, w, threads, ctas, smem, s)
                         : launch_k(row_model_kernel<H, false>, L, w, threads, ctas, smem, s);
+  if (L.spread_mode == 3 && L.qmode) return launch_k(row_adjoint_pairs_kernel<H, true, true>, L, w, threads, ctas, smem, s);
   if (L.spread_mode == 3)
     return zf ? launch_k(row_adjoint_pairs_kernel<H, true>, L, w, threads, ctas, smem, s)
               : launch_k(row_adjoint_pairs_kernel<H, false>, L, w, threads, ctas, smem, s);
@@ -51,12 +52,13 @@ static cudaError_t adj_h(const RowLaunch& L, const WindowPoly& w, int threads, i
 }
 
 // kind: 0 forward, 1 adjoint, 2 adjoint with the pair spread, 3 forward (paired layout), 4 forward model,
-// 5 forward model in units of two rows
+// 5 forward model in units of two rows, 6 forward model by node pairs
 template <int H>
 static int occ_h(int kind, int threads, size_t smem, bool zf) {
   if (kind == 2)
     return zf ? occ_k(row_adjoint_pairs_kernel<H, true>, threads, smem)
               : occ_k(row_adjoint_pairs_kernel<H, false>, threads, smem);
+  if (kind == 6) return occ_k(row_adjoint_pairs_kernel<H, true, true>, threads, smem);
   if (kind == 4) return occ_k(row_model_kernel<H, false>, threads, smem);
   if (kind == 5) return occ_k(row_model_kernel<H, true>, threads, smem);
   if (kind == 3) return occ_k(row_forward_kernel<H, false, true>, threads, smem);

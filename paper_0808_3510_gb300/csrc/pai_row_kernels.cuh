@@ -1157,23 +1157,30 @@ struct PairSrc {
   float2 S;         // |K_lat / 2 pi|^2 as float-float
   bool mirror;      // the row has -nu nodes below the Nyquist entry
 };
+// The depth index of node pair 0: forward models have a pair at depth frequency 0 too.
+template <bool Q>
+constexpr int kFirstPair = Q ? 0 : 1;
 
-// Node pair i of a row: the nodes +-x of one depth index l = i + 1,
+// Node pair i of a row: the nodes +-x of one depth index l = i + kFirstPair,
 // x = j0 + fr, and their values Q+ = qp, Q- = qn: the
 // input times the weight and the transpose of the node's phase, e^{+i pi nu}
-// for +x and its conjugate for -x.
-template <bool ZF>
+// for +x and its conjugate for -x.  Q (forward model): both nodes carry c_l / 2
+// (wscale holds 1 / (2 n_lat nz)).
+template <bool ZF, bool Q>
 __device__ __forceinline__ void pair_node(const RowProblem& P, const PairSrc& src, int i, int& j0, float& fr,
                                           float2& qp, float2& qn) {
   const int nzh = P.nz >> 1;
-  const int lp = i + 1;
+  const int lp = i + kFirstPair<Q>;
   const float4 zt = __ldg(&P.zt[lp]);
   float rx;
   node_position(src.S, zt, P.B2hi, P.B2lo, j0, fr, rx);
   const float2 ph = node_phase(j0, fr, P.nt, P.M, P.nt_over_M);
   float2 yp, yn;  // inputs of the two nodes, real weights applied
   const float wt = P.wscale * zt.z * rx;
-  if (lp == nzh) {
+  if (Q) {
+    const float2 y = src.a[lp];
+    yp = yn = make_float2(P.wscale * y.x, P.wscale * y.y);
+  } else if (lp == nzh) {
     // Nyquist: both nodes carry half the l = -nz/2 input
     float2 y = src.a[lp];
     if (!ZF && src.mirror) {
@@ -1544,13 +1551,13 @@ __device__ __forceinline__ void band_end(const BandPart<H>& b, Band& band, int l
 // 221 us, 666x1500 (M = 4096) 21.6 -> 18.3 us.  Spreading two pairs per lane as
 // the forward model does paid at 256^3 (216 us) but not for longer rows or wider
 // windows (105 and 19.6 us), whose weights leave the registers.
-template <int H, bool ZF>
+template <int H, bool ZF, bool Q>
 __device__ __forceinline__ bool adjoint_band(const RowProblem& P, const WindowPoly& W, int row, bool valid, int lane,
                                              float2* X, Band& band) {
   PairSrc src{nullptr, nullptr, make_float2(0.f, 0.f), true};
   int np = 0;
   if (valid) {
-    np = P.nz >> 1;
+    np = (P.nz >> 1) + 1 - kFirstPair<Q>;
     if (ZF) {
       src.a = P.fh + (size_t)row * P.zstride;
       src.S = P.rowS[row];
@@ -1566,7 +1573,7 @@ __device__ __forceinline__ bool adjoint_band(const RowProblem& P, const WindowPo
   band_begin<H, true>(part, band, reinterpret_cast<char*>(X), P.band_ps, np, lane, P.tpr, [&](int i) {
     int j0;
     float fr, rx;
-    node_position(src.S, __ldg(&P.zt[i + 1]), P.B2hi, P.B2lo, j0, fr, rx);
+    node_position(src.S, __ldg(&P.zt[i + kFirstPair<Q>]), P.B2hi, P.B2lo, j0, fr, rx);
     return j0;
   });
   // chunks: uniform over the warp (rows sharing a warp have equal counts, or none)
@@ -1577,7 +1584,7 @@ __device__ __forceinline__ bool adjoint_band(const RowProblem& P, const WindowPo
     int j0 = 0;
     float fr = 0.5f;
     float2 qp = make_float2(0.f, 0.f), qn = qp;
-    if (act) pair_node<ZF>(P, src, i, j0, fr, qp, qn);
+    if (act) pair_node<ZF, Q>(P, src, i, j0, fr, qp, qn);
     const int c = j0 - H + 1;  // first cell
     const BandTaps<true> tp(band, c - band.lo, part.spill_w + ((c - part.lo_w) << 4), part.hi_prev + 1 - c);
     band_spread<H, true>(W, tp, j0, fr, Cell<true>{make_float4(qp.x, qp.y, qn.x, qn.y)}, act, part.gw);
@@ -1588,8 +1595,10 @@ __device__ __forceinline__ bool adjoint_band(const RowProblem& P, const WindowPo
 }
 
 // The adjoint row kernel with the pair spread (spread mode 3), a kernel of its
-// own so that its register allocation does not carry the other schemes.
-template <int H, bool ZF>
+// own so that its register allocation does not carry the other schemes.  Q: the
+// discrete forward model by node pairs, for windows that row_model_kernel is not
+// used for (see there) and rows that do not fit it.
+template <int H, bool ZF, bool Q = false>
 __global__ void __launch_bounds__(1024) row_adjoint_pairs_kernel(RowLaunch L, WindowPoly W) {
   extern __shared__ __align__(16) float2 smem[];
   __shared__ int s_item;
@@ -1604,7 +1613,7 @@ __global__ void __launch_bounds__(1024) row_adjoint_pairs_kernel(RowLaunch L, Wi
     const bool valid = row < P.rows;
     float2* X = smem + slot * P.band_slot;
     Band band;
-    const bool mirror = adjoint_band<H, ZF>(P, W, row, valid, lane, X, band);
+    const bool mirror = adjoint_band<H, ZF, Q>(P, W, row, valid, lane, X, band);
     const float scale = (valid && !ZF && mirror) ? 0.5f : 1.0f;
     float2* dst = const_cast<float2*>(P.pt) + (size_t)(valid ? row : 0) * nt;
     fft_inverse_crop<true>(X, M, P.mshift, nt, lane, tpr, L.tw, L.Mmax >> P.mshift, dst, P.prescale, scale, valid,
@@ -1669,7 +1678,12 @@ __device__ __forceinline__ void model_last(const float2* X, int M, int nt, int l
 //   g_n = t_n V[n] + conj(t_n) V[M - n],   t_n = s_n e^{-i pi n / (2M)},
 // s_n the window's prescale over the doubled interval.  Against the node pairs
 // of the adjoint (two nodes with phases per index) this halves the values
-// spread and drops a sine and cosine per node.
+// spread and drops a sine and cosine per node.  The
+// window's error falls on other samples than with the node pairs (it is largest
+// towards n = nt, theirs towards both ends), so only windows whose error is below
+// rounding take this kernel; the others keep the pairs in band grids
+// (row_adjoint_pairs_kernel: truncated sinc, 12 taps, 128^3 1369 us a call, 2683
+// with the pair warps and the stored box before both).
 //
 // PAIR (3-D): rows k1 and -k1 have the same |K| and so the same nodes; a unit
 // of 2 tpr threads spreads both rows' values with one set of weights into
