@@ -1542,9 +1542,10 @@ __device__ __forceinline__ void band_end(const BandPart<H>& b, Band& band, int l
 // pair's values are formed right before they are spread (no list in shared
 // memory).
 //
-// What bounds it: instruction issue (57 % of the slots) and shared-memory
-// accesses (69 % of their peak; 32 bytes per tap and pair) about equally, behind
-// them the latency of the tap chain; 64 registers at 32 warps per SM measured
+// What bounds it: shared-memory accesses (32 bytes per tap and pair; 256^3: 81 %
+// of their peak, 38 % of the wavefronts bank conflicts, issue slots 55 %), in
+// long rows with fewer CTAs also the latency of the tap chain and the barriers
+// (2048x4096: 61 % and 42 %); 64 registers at 32 warps per SM measured
 // best (56: +6 %, 90 and half the warps: +16 %).  The lists, run sums and float
 // atomics it replaced held one CTA per SM for long rows and serialised on equal
 // cells: 2048x4096 (M = 8192, H = 8) 126 -> 91 us, 256^3 (M = 1024, H = 6) 224 ->
@@ -1678,19 +1679,19 @@ __device__ __forceinline__ void model_last(const float2* X, int M, int nt, int l
 //   g_n = t_n V[n] + conj(t_n) V[M - n],   t_n = s_n e^{-i pi n / (2M)},
 // s_n the window's prescale over the doubled interval.  Against the node pairs
 // of the adjoint (two nodes with phases per index) this halves the values
-// spread and drops a sine and cosine per node.  The
-// window's error falls on other samples than with the node pairs (it is largest
-// towards n = nt, theirs towards both ends), so only windows whose error is below
-// rounding take this kernel; the others keep the pairs in band grids
-// (row_adjoint_pairs_kernel: truncated sinc, 12 taps, 128^3 1369 us a call, 2683
+// spread and drops a sine and cosine per node.  The window's error falls on other
+// samples than with the node pairs, so only windows whose error is below rounding
+// take this kernel; the others keep the pairs in band grids
+// (row_adjoint_pairs_kernel; truncated sinc, 12 taps, 128^3: 1369 us a call, 2683
 // with the pair warps and the stored box before both).
 //
 // PAIR (3-D): rows k1 and -k1 have the same |K| and so the same nodes; a unit
 // of 2 tpr threads spreads both rows' values with one set of weights into
 // 16-byte cells, then transforms one row with each half of its threads.
 //
-// What bounds it: shared-memory accesses (79 % of their peak) and instruction
-// issue (64 % of the slots), about a third of it node positions and weights.
+// What bounds it: shared-memory accesses and instruction issue (128^3: 81 % of
+// their peak and 65 % of the slots; 2048x4096: 63 and 60 %, and barriers), about a
+// third of the issue node positions and weights.
 // 128^3 in its 512^3 box (131 584 rows, M = 512): 1264 us with the node pairs of
 // the adjoint and their lists, 957 us with them in band grids, 675 us as this
 // kernel, 604 us with two nodes per lane (band_spread2); 2048x4096 in 8192^2
