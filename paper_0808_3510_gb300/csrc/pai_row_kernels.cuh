@@ -682,25 +682,38 @@ __device__ __forceinline__ void fft_last_crop(const float2* X, int M, int nt, in
 // kept, and only those 8 outputs are computed: with w = e^{+2 pi i/16},
 // A = inverse DFT8 of the even inputs and B of the odd,
 // Y[t] = A[t] + w^t B[t] (t = 0..3) and Y[t+8] = A[t] - w^t B[t] (t = 4..7).
-// BAND: the first pass reads the band grid.  (Otherwise one pad per 32, so
-// that the list spreads' rows and node lists fit in shared memory up to the
-// sizes they always did.)
+// BAND: the first pass reads the band grid.  Otherwise (list spreads) the
+// remaining radix comes first and radix 16 last: their kernel holds three spreads
+// and has no registers left for the three other last passes (tap phases with
+// linear interpolation at M = 8192: 92.5 us, 105 with them); and one pad per 32,
+// so that rows and node lists fit in shared memory up to the sizes they always did.
 template <bool BAND>
 __device__ __forceinline__ void fft_inverse_crop(float2* X, int M, int mshift, int nt, int lane, int tpr,
                                                  const float2* __restrict__ tw, int twstride, float2* dst,
                                                  const float* __restrict__ prescale, float scale, bool valid,
                                                  const Band& band) {
   constexpr int PS = BAND ? 4 : 5;
-  if (BAND) fft_first_pass_band(X, M, lane, tpr, band);
-  else fft_pass<16, true, kLayoutPadded, 2, PS>(X, M, 1, lane, tpr, tw, twstride);
-  int Ns = 16;
   const int r0 = mshift & 3;
+  int Ns = 1;
+  if (BAND) {
+    fft_first_pass_band(X, M, lane, tpr, band);
+    Ns = 16;
+  } else if (r0 == 3) {
+    fft_pass<8, true, kLayoutPadded, 2, PS>(X, M, 1, lane, tpr, tw, twstride);
+    Ns = 8;
+  } else if (r0 == 2) {
+    fft_pass<4, true, kLayoutPadded, 2, PS>(X, M, 1, lane, tpr, tw, twstride);
+    Ns = 4;
+  } else if (r0 == 1) {
+    fft_pass<2, true, kLayoutPadded, 2, PS>(X, M, 1, lane, tpr, tw, twstride);
+    Ns = 2;
+  }
   while (Ns * 16 < M) {
     fft_pass<16, true, kLayoutPadded, 2, PS>(X, M, Ns, lane, tpr, tw, twstride);
     Ns <<= 4;
   }
   if (!valid) return;
-  if (r0 != 0) {
+  if (BAND && r0 != 0) {
     if (r0 == 3) fft_last_crop<8, PS>(X, M, nt, lane, tpr, tw, twstride, dst, prescale, scale);
     else if (r0 == 2) fft_last_crop<4, PS>(X, M, nt, lane, tpr, tw, twstride, dst, prescale, scale);
     else fft_last_crop<2, PS>(X, M, nt, lane, tpr, tw, twstride, dst, prescale, scale);
