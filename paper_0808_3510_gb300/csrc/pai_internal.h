@@ -31,11 +31,14 @@ inline cudaError_t launch_kernel(void (*k)(P...), dim3 grid, dim3 block, size_t 
   c.numAttrs = pdl ? 1 : 0;
   return cudaLaunchKernelEx(&c, k, P(args)...);
 }
-// Allows `smem` bytes of dynamic shared memory; up to 48 KB (with the static part) need no call.
+// Allows `smem` bytes of dynamic shared memory; up to 48 KB (with the static part) need no call.  The limit belongs to
+// the function, not to the launch: it is always set to the same value (226 of the 227 KB, the rest for static shared
+// memory), so that a thread with a smaller plan does not lower it between another's call and launch.
 template <typename K>
 inline cudaError_t allow_smem(K* kernel, size_t smem) {
   if (smem <= 47 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr size_t kLimit = 226 * 1024;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem > kLimit ? smem : kLimit));
 }
 #ifdef __CUDACC__
 // First statement of a kernel: waits for the previous one.  What an earlier
