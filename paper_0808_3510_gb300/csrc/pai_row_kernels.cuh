@@ -685,7 +685,7 @@ __device__ __forceinline__ void fft_last_crop(const float2* X, int M, int nt, in
 // BAND: the first pass reads the band grid.  Otherwise (list spreads) the
 // remaining radix comes first and radix 16 last: their kernel holds three spreads
 // and has no registers left for the three other last passes (tap phases with
-// linear interpolation at M = 8192: 92.5 us, 105 with them); and one pad per 32,
+// linear interpolation at M = 8192: 100.5 us, 105 with them); and one pad per 32,
 // so that rows and node lists fit in shared memory up to the sizes they always did.
 template <bool BAND>
 __device__ __forceinline__ void fft_inverse_crop(float2* X, int M, int mshift, int nt, int lane, int tpr,
