@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include <utility>
@@ -94,7 +95,9 @@ struct WindowPoly {
 // One reconstruction problem as the row kernels see it.  Lateral axes are
 // (n1, n2) with n2 the axis halved by the real-to-complex lateral FFT:
 // 2-D: (1, nx); 3-D: (nx, ny).  Row r = i1 * (n2/2 + 1) + i2.
-struct RowProblem {
+struct alignas(128) RowProblem {
+  // what the forward kernel reads, in the record's first 128 bytes (one cache line; the records of a batch compete for
+  // L1 with its rows: 64 problems' row kernel 1.2189 ms with them spread over two lines, 1.2154 ms so)
   const float2* pt;        // lateral spectrum rows [rows][nt] (fwd in / adj out)
   float2* fh;              // image half spectrum [n1*n2][lz] (fwd out / adj in)
   const float* prescale;   // [nt] window prescale incl. all constant factors
@@ -103,14 +106,19 @@ struct RowProblem {
   int nt, M, nz, lz;
   int n1, n2, rows;
   int tpr;                 // threads per row in the FFT = M / kElemsPerThread
-  int rpc;                 // rows per CTA work item
-  int slot;                // complex values per row slot in shared memory (row_slot_stride(M)): band spreads
-  int slot32;              // the same with one pad per 32: forward kernel and the adjoint's list spreads
+  int slot32;              // complex values per row slot in shared memory with one pad per 32 (row_slot_stride(M, 5)):
+                           // forward kernel and the adjoint's list spreads
+  int mshift;              // log2(M)
   float B2hi, B2lo;        // (M c dt)^2 as float-float: node x = B sqrt(S + az)
   float wscale;            // 2 c dt/dz * B / (n1 n2 nz): W = wscale * kz / x
   float nt_over_M;         // for the node phase
-  int mshift;              // log2(M)
   int method;              // PAI_METHOD_*
+  int paired;              // 2-D, forward: pt holds Z[k][m] (k < nx = n2, m < nt/2, row stride nt/2), the
+                           // lateral DFT of the sample pairs p[x][2m] + i p[x][2m+1]; the forward row kernel
+                           // separates row k's samples from Z[k] and Z[nx - k]
+  int rpc;                 // rows per CTA work item
+  // adjoint and forward model
+  int slot;                // complex values per row slot with one pad per 16 (row_slot_stride(M)): band spreads
   int qmode;               // adjoint kernel evaluates the discrete forward model (depth-row layout only)
   int zstride;             // depth-row layout: complex values from one row to the next (nz; in qmode
                            // the rows hold c_j, j = 0..nz/2, nz/2 + 2 values apart)
@@ -118,10 +126,8 @@ struct RowProblem {
   int model_ps, model_slot;  // the same for the forward-model row kernel (per unit of one or two rows)
   int model_dense;           // neighbouring nodes are at most two cells apart there
   const float2* model_tab;   // forward-model row kernel: [nt] prescale times e^{-i pi n / (2M)}
-  int paired;              // 2-D, forward: pt holds Z[k][m] (k < nx = n2, m < nt/2, row stride nt/2), the
-                           // lateral DFT of the sample pairs p[x][2m] + i p[x][2m+1]; the forward row kernel
-                           // separates row k's samples from Z[k] and Z[nx - k]
 };
+static_assert(offsetof(RowProblem, rpc) + sizeof(int) <= 128 && sizeof(RowProblem) <= 256, "RowProblem layout");
 
 struct WorkItem {
   int problem;  // index into the RowProblem array
