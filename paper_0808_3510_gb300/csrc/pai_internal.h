@@ -96,8 +96,8 @@ struct WindowPoly {
 // (n1, n2) with n2 the axis halved by the real-to-complex lateral FFT:
 // 2-D: (1, nx); 3-D: (nx, ny).  Row r = i1 * (n2/2 + 1) + i2.
 struct alignas(128) RowProblem {
-  // what the forward kernel reads, in the record's first 128 bytes (one cache line; the records of a batch compete for
-  // L1 with its rows: 64 problems' row kernel 1.2189 ms with them spread over two lines, 1.2154 ms so)
+  // what the row kernels read per item, in the record's first 128 bytes (one cache line; the records of a batch compete
+  // for L1 with its rows: 64 problems' row kernel 1.219 ms with them spread over two lines, 1.211 ms so)
   const float2* pt;        // lateral spectrum rows [rows][nt] (fwd in / adj out)
   float2* fh;              // image half spectrum [n1*n2][lz] (fwd out / adj in)
   const float* prescale;   // [nt] window prescale incl. all constant factors
@@ -116,18 +116,19 @@ struct alignas(128) RowProblem {
   int paired;              // 2-D, forward: pt holds Z[k][m] (k < nx = n2, m < nt/2, row stride nt/2), the
                            // lateral DFT of the sample pairs p[x][2m] + i p[x][2m+1]; the forward row kernel
                            // separates row k's samples from Z[k] and Z[nx - k]
-  int rpc;                 // rows per CTA work item
   // adjoint and forward model
   int slot;                // complex values per row slot with one pad per 16 (row_slot_stride(M)): band spreads
-  int qmode;               // adjoint kernel evaluates the discrete forward model (depth-row layout only)
   int zstride;             // depth-row layout: complex values from one row to the next (nz; in qmode
                            // the rows hold c_j, j = 0..nz/2, nz/2 + 2 values apart)
   int band_ps, band_slot;  // adjoint pair spread: cells per phase of the band grid, complex values per row slot
   int model_ps, model_slot;  // the same for the forward-model row kernel (per unit of one or two rows)
-  int model_dense;           // neighbouring nodes are at most two cells apart there
+  // beyond the first 128 bytes
+  int model_dense;           // neighbouring nodes are at most two cells apart in the forward model
+  int qmode;               // adjoint kernel evaluates the discrete forward model (depth-row layout only)
   const float2* model_tab;   // forward-model row kernel: [nt] prescale times e^{-i pi n / (2M)}
+  int rpc;                 // rows per CTA work item
 };
-static_assert(offsetof(RowProblem, rpc) + sizeof(int) <= 128 && sizeof(RowProblem) <= 256, "RowProblem layout");
+static_assert(offsetof(RowProblem, model_slot) + sizeof(int) <= 128 && sizeof(RowProblem) <= 256, "RowProblem layout");
 
 struct WorkItem {
   int problem;  // index into the RowProblem array
